@@ -115,6 +115,25 @@ bool encode_row_map(void* base, size_t elem, int Lx, int Ly, int cols, int rows,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same for the stream kernel, whose advect warps each stage the four planes
+// k = 4 group + q of one sign quadrant q: a 4-D tensor (x, q, group, row) read
+// in boxes of `cols` columns x 1 quadrant x 4 groups x `rows` rows.
+bool encode_quadrant_map(void* base, size_t elem, int Lx, int Ly, int cols, int rows,
+                         CUtensorMap* out) {
+  const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc || Lx < cols || Ly < rows) return false;
+  const cuuint64_t plane = (cuuint64_t)Lx * (cuuint64_t)Ly * elem;
+  const cuuint64_t dims[4] = {(cuuint64_t)Lx, 4, 4, (cuuint64_t)Ly};
+  const cuuint64_t strides[3] = {plane, 4 * plane, (cuuint64_t)Lx * elem};
+  const cuuint32_t box[4] = {(cuuint32_t)cols, 1, 4, (cuuint32_t)rows};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  const CUtensorMapDataType type =
+      elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+  return enc(out, type, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // f [16][Ly][Lx] as a 3-D tensor ordered (x, row, plane), written in tiles of
 // TW columns x RPI rows x 16 planes: a tile is [16][RPI][TW] in shared memory
 // (the collision's plane-major output tile).  False when the encoder is
@@ -198,6 +217,7 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   a.om2 = (T)(0.5 * om);
   a.om6 = (T)(om / 6.0);
   a.rho_ext = (T)p.rho_ext;
+  a.irho_ext = (T)(p.rho_ext != 0.0 ? 1.0 / p.rho_ext : 0.0);
   const int Lmin = p.Lx < p.Ly ? p.Lx : p.Ly;
   const double rbc = Lmin / 2.0 - 1.0 / (2.0 * p.ds);
   a.rbc2 = (T)(rbc > 0 ? rbc * rbc : 0.0);
@@ -206,6 +226,15 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   a.err = h->d_err;
   a.xlo = (T)std::sqrt(3.0 - std::sqrt(6.0));
   a.xhi = (T)std::sqrt(3.0 + std::sqrt(6.0));
+  a.lo2 = (T)(3.0 - std::sqrt(6.0));
+  a.hi2 = (T)(3.0 + std::sqrt(6.0));
+  const double ps = 0.5 * (p.T - 1.0);
+  a.ps = (T)ps;
+  a.p00 = (T)(-2.0 * om * ps);
+  a.p10 = (T)(om - 4.0 * om * ps);
+  a.pg = (T)(3.0 - 2.0 * p.T);
+  a.p20 = (T)(om * ps);
+  a.p30 = (T)(-2.0 * om / 3.0);
   for (int grp = 0; grp < 4; ++grp) {
     const int k = 4 * grp;
     const double x2 = h->xi[k][0] * h->xi[k][0] + h->xi[k][1] * h->xi[k][1];
@@ -242,6 +271,8 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
     v.ax = (T)(2.0 * lam * hx);
     v.by0 = (T)(-2.0 * lam * hy * (1.0 - cx));
     v.by1 = (T)(-2.0 * lam * hy * cx);
+    v.qy0 = (T)((1.0 - cy) * (1.0 - cx));
+    v.qy1 = (T)((1.0 - cy) * cx);
     v.gbot = (T)(gb[k] - h->w[k] * rr);
     v.gtop = (T)(gt[k] - h->w[k] * rr);
     // Eq. (ereg): w [ H2:A2 / 2! + H3:A3 / 3! ] over the independent components
@@ -324,6 +355,24 @@ void finish_diag(const DiagAcc& acc, bool full, lbm_diag* out) {
   }
 }
 
+// Rows per work item.  A persistent CTA works through its items one after the
+// other; an item of r rows costs r rows and the pipeline's warm-up of 8, and the
+// launch ends with the CTA that has the most items: the block that minimises
+// rounds x (r + 8), never under 16 rows.
+long long pick_row_block(int Ly, int nstrip, long long grid) {
+  long long best = 16, cost = 0;
+  for (long long rb = 16; rb <= 1024; rb += 4) {
+    const long long items = (Ly + rb - 1) / rb * nstrip;
+    const long long c = (items + grid - 1) / grid * (rb + 8);
+    if (cost == 0 || c < cost) {
+      cost = c;
+      best = rb;
+    }
+    if (rb >= Ly) break;
+  }
+  return best;
+}
+
 int check_device_error(lbm_handle* h) {
   unsigned int e = 0;
   if (cudaMemcpyAsync(&e, h->d_err, sizeof(e), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
@@ -398,12 +447,24 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
   // values, 8 for half), output tiles stored by tensor stores
   std::memset(h->tmap, 0, sizeof(h->tmap));
   bool tin = (p->Lx % (h->elem == 2 ? 8 : 4)) == 0, tout = tin;
-  const int scol = h->elem == 2 ? scol_of<__half>() : scol_of<float>();
+  tin = tin && p->Lx >= (h->elem == 2 ? 72 : 68);
+  const int last = (p->Lx - 1) / TW;  // the last strip
   for (int i = 0; i < 2; ++i) {
-    tin = tin && encode_row_map(h->f[i], h->elem, p->Lx, p->Ly, scol, RPI, &h->tmap[i].m[0]) &&
-          encode_row_map(h->f[i], h->elem, p->Lx, p->Ly, scol, 1, &h->tmap[i].m[1]);
-    tout = tout && encode_tile_map(h->f[1 - i], h->elem, p->Lx, p->Ly, &h->tmap[i].m[2]);
+    if (h->elem == 8) {
+      tin = tin && encode_row_map(h->f[i], 8, p->Lx, p->Ly, scol_of<double>(), RPI, &h->tmap[i].m[0]) &&
+            encode_row_map(h->f[i], 8, p->Lx, p->Ly, scol_of<double>(), 1, &h->tmap[i].m[1]);
+      tout = tout && encode_tile_map(h->f[1 - i], 8, p->Lx, p->Ly, &h->tmap[i].m[2]);
+    } else {
+      // columns of a strip's staging, and of the runs at the left and right seam
+      const int soff = h->elem == 2 ? StreamLayout<__half>::SOFF : StreamLayout<float>::SOFF;
+      const int scol = REG + 2 * soff, nl = XOFF + soff, nr = p->Lx - (last * TW - XOFF - soff);
+      const int cols[5] = {scol, nl, scol - nl, nr, scol - nr};
+      for (int m = 0; m < 5; ++m)
+        tin = tin && (cols[m] <= 0 || cols[m] > scol ||  // (the last strip ends at the seam)
+                      encode_quadrant_map(h->f[i], h->elem, p->Lx, p->Ly, cols[m], SR, &h->tmap[i].m[m]));
+    }
   }
+  tin = tout = tin && tout;
   h->vec = tin;  // else every strip stages by per-thread loads
 
   // launch geometry: strips of TW output columns, rows split evenly over a
@@ -421,20 +482,8 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
     lbm_destroy(h);
     return LBM_ERR_CUDA;
   }
-  // work items: row blocks of up to 256 rows x strips; blocks shrink (down to
-  // 96 rows, where the 7-row pipeline warm-up still costs < 8 %) when a
-  // lattice would leave the grid with fewer than ~3 items per CTA.  A lattice
-  // too small to give every CTA one 96-row item is latency-bound: its blocks
-  // shrink further (down to 16 rows), trading warm-up work for a shorter row
-  // loop per CTA.
-  const long long rows_total = (long long)h->nstrip * p->Ly;
   const long long grid_max = (long long)nsm * occ;
-  long long rb = rows_total / (3 * grid_max);
-  rb = rb < 96 ? 96 : (rb > 256 ? 256 : rb);
-  if (rows_total < 96 * grid_max) {
-    const long long fill = (rows_total + grid_max - 1) / grid_max;
-    rb = fill < 16 ? 16 : fill;
-  }
+  const long long rb = pick_row_block(p->Ly, h->nstrip, grid_max);
   h->row_block = (int)rb;
   const long long items = (long long)((p->Ly + rb - 1) / rb) * h->nstrip;
   h->grid = (int)(items < grid_max ? items : grid_max);

@@ -285,6 +285,8 @@ cudaError_t launch_hist(const AuxArgs& a, const void* f, int nbins, double lo, d
 }
 
 size_t step_smem_bytes(size_t stage_elem, size_t elem) {
+  if (elem == 4)
+    return stage_elem == 2 ? StreamSmem<__half>::bytes() : StreamSmem<float>::bytes();
   const size_t elems = (size_t)FROWS * FRS + 4 * (size_t)MROWS * MP;  // f*, drho, ux, uy, phi
   // + 128 bytes to align the staging ring (which also holds the output tiles)
   // for tensor copies; the fused diagnostics' bubble-site sums, the staging

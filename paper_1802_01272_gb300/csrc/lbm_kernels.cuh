@@ -9,7 +9,7 @@
 // relaxation (optionally regularised, Eq. ereg), and the density reservoir of
 // Sec. III A.
 //
-// Kernel layout (step_kernel): a CTA owns a strip of TW = 56 output columns
+// FP32 arithmetic: step_stream.cuh.  FP64 kernel layout (step_kernel): a CTA owns a strip of TW = 56 output columns
 // [56 s, 56 s + 56) and streams down a range of rows, 4 rows per iteration.
 // Its 256 threads are (velocity k, group g of four columns) over a 64-column
 // region [56 s - 4, 56 s + 60): the strip, the two columns of rho* halo the
@@ -77,6 +77,7 @@ struct VelConst {
   T cx, cy;                 // Courant numbers |xi_x| dt/ds, |xi_y| dt/ds
   T ax;                     // lam |xi_x| (1 - cx): weight of the x-difference of half-limited S^x
   T by0, by1;               // -lam |xi_y| (1 - cy) (1 - cx), -lam |xi_y| (1 - cy) cx (S^y terms)
+  T qy0, qy1;               // (1 - cy) (1 - cx), (1 - cy) cx: the same per unit of cy
   T gbot, gtop;             // wall ghost-row values (storage variable)
   T r2xx, r2xy, r2yy, r3xxx, r3xxy, r3xyy, r3yyy;  // Eq. (ereg) weights, 1/n! folded in
 };
@@ -111,20 +112,27 @@ struct StepArgs {
   // q(+-1, b) - q(-+1, b) for |b| = 0, 1, 2 and of q(+-2, b) - q(-+2, b),
   // (-1, -1/18, 1/18, 1/4, 1/9, 1/72) kappa dt/ds^3
   T kw[6];
-  T rho_ext, rbc2, cxc, cyc;
+  T rho_ext, irho_ext, rbc2, cxc, cyc;
   unsigned int* err;         // bit 0: non-finite or non-positive rho; bit 1: a wait timed out
   int tma_in;               // the tensor maps describe fin (interior strips stage by tensor copies)
   int tma_out;              // the store maps describe fout (tiles leave by tensor stores)
   T xlo, xhi;               // |xi| components sqrt(3 - sqrt 6), sqrt(3 + sqrt 6)
+  T lo2, hi2;               // their squares
+  // constants of the collision polynomial, w = dt/tau: s = (T - 1)/2, -2 w s, w - 4 w s,
+  // 3 - 2 T, w s, -2 w / 3
+  T ps, p00, p10, pg, p20, p30;
   ClassConst<T> cls[4];     // groups (lo,lo), (hi,lo), (lo,hi), (hi,hi)
   VelConst<T> v[16];
 };
 
-// f^n as a 3-D tensor (x, plane, row): m[0] loads boxes of scol_of<ST>()
-// columns x 16 planes x RPI rows of fin, m[1] single rows; f^{n+1} as (x, row, plane):
-// m[2] stores tiles of TW columns x RPI rows x 16 planes into fout.
+// Tensor maps of f^n.  FP64: as a 3-D tensor (x, plane, row), m[0] loads boxes of
+// scol_of<ST>() columns x 16 planes x RPI rows, m[1] single rows; f^{n+1} as (x,
+// row, plane): m[2] stores tiles of TW columns x RPI rows x 16 planes.  FP32 and
+// FP16: as a 4-D tensor (x, sign quadrant, group, row), boxes of one quadrant's
+// four planes x SR rows: m[0] all columns of a strip's staging, m[1] and m[2] the
+// two runs of the strip at the left x seam, m[3] and m[4] of that at the right.
 struct RowMaps {
-  CUtensorMap m[3];
+  CUtensorMap m[5];
 };
 
 constexpr int MAXB = 12;  // lattices per batched launch (kernel parameter space)
@@ -384,14 +392,10 @@ __device__ __forceinline__ void advect_row(AdvState<T>& s, const ST* srow, const
   }
 }
 
-// ------------------------------------------- packed FP32 advection (FP32 and FP16 storage)
-// The same row update on column pairs (0, 1) and (2, 3) held as float2: every
-// operation whose operands are whole pairs runs as one packed FP32x2
-// instruction (sm_100+), which issues once for two lanes' worth of work; the
-// jumps R^x (pairs shifted by one column), the limiters (min/max have no
-// packed form) and the neighbour-shifted terms stay scalar.  Numerically each
-// component is the scalar operation (round to nearest), except h^x, taken as
-// (f(i) - f(i-2))/4 for s_x > 0 (the same quantity as (R^x(i) + R^x(i-1))/4).
+// ------------------------------------------------------- pairs of values
+// Two neighbouring columns or nodes as one value: in FP32 every operation on
+// whole pairs is one packed FP32x2 instruction (sm_100+, round to nearest),
+// which issues once for two lanes' worth of work.
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -435,32 +439,6 @@ __device__ __forceinline__ float mc_half(float R, float Ru, float h) {
   }
 }
 
-struct AdvState2 {
-  float2 Fp[2], Ryp[2], Syp[2], Z1[2], Z2[2], pend[2];  // as AdvState, column pairs
-};
-
-// per-thread constant pairs of the packed row update
-struct VelPairs {
-  float2 ncx, nax, cy, by0, q;  // (-/+)c_x (sign of -s_x), -ax, c_y, by0, 1/4
-  float by1;
-};
-template <int SX>
-__device__ __forceinline__ VelPairs vel_pairs(const VelConst<float>& c) {
-  VelPairs v;
-  v.ncx = dup2(SX > 0 ? -c.cx : c.cx);
-  v.nax = dup2(-c.ax);
-  v.cy = dup2(c.cy);
-  v.by0 = dup2(c.by0);
-  v.q = dup2(0.25f);
-  v.by1 = c.by1;
-  return v;
-}
-
-template <typename ST>
-__device__ __forceinline__ float2 sload2(const ST* p) {
-  if constexpr (sizeof(ST) == 4) return *reinterpret_cast<const float2*>(p);
-  else return __half22float2(*reinterpret_cast<const __half2*>(p));
-}
 template <typename ST>
 __device__ __forceinline__ void sload4p(const ST* p, float2& a, float2& b) {
   if constexpr (sizeof(ST) == 4) {
@@ -474,121 +452,14 @@ __device__ __forceinline__ void sload4p(const ST* p, float2& a, float2& b) {
   }
 }
 
-template <int SX, int SY, int ORDER, int LIM, typename ST>
-__device__ __forceinline__ void advect_row2(AdvState2& s, const ST* srow, const VelPairs& c,
-                                            float* out) {
-  float2 B0, B1;  // columns (0, 1), (2, 3)
-  sload4p<ST>(srow, B0, B1);
-  float2 Z[2];
-  if constexpr (SX > 0) {
-    const float2 A = sload2<ST>(srow - 2);  // columns (-2, -1)
-    const float R_1 = A.y - A.x, R0 = B0.x - A.y, R1 = B0.y - B0.x;
-    const float R2 = B1.x - B0.y, R3 = B1.y - B1.x;
-    const float2 X01 = fma2(c.ncx, make_float2(R0, R1), B0);
-    const float2 X23 = fma2(c.ncx, make_float2(R2, R3), B1);
-    if constexpr (ORDER == 2) {
-      const float2 h01 = mul2(c.q, sub2(B0, A)), h23 = mul2(c.q, sub2(B1, B0));
-      const float S0 = mc_half<LIM>(R0, R_1, h01.x), S1 = mc_half<LIM>(R1, R0, h01.y);
-      const float S2 = mc_half<LIM>(R2, R1, h23.x), S3 = mc_half<LIM>(R3, R2, h23.y);
-      const float S4 = shfl_dn1(S0);
-      Z[0] = fma2(c.nax, make_float2(S1 - S0, S2 - S1), X01);
-      Z[1] = fma2(c.nax, make_float2(S3 - S2, S4 - S3), X23);
-    } else {
-      Z[0] = X01;
-      Z[1] = X23;
-    }
-  } else {
-    const float a = from_store<ST, float>(srow[-1]), e = from_store<ST, float>(srow[4]);
-    const float R0 = B0.x - a, R1 = B0.y - B0.x, R2 = B1.x - B0.y;
-    const float R3 = B1.y - B1.x, R4 = e - B1.y;
-    const float2 X01 = fma2(c.ncx, make_float2(R1, R2), B0);
-    const float2 X23 = fma2(c.ncx, make_float2(R3, R4), B1);
-    if constexpr (ORDER == 2) {
-      const float S0 = mc_half<LIM>(R0, R1, 0.25f * (R0 + R1));
-      const float S1 = mc_half<LIM>(R1, R2, 0.25f * (R1 + R2));
-      const float S2 = mc_half<LIM>(R2, R3, 0.25f * (R2 + R3));
-      const float S3 = mc_half<LIM>(R3, R4, 0.25f * (R3 + R4));
-      const float S4 = shfl_dn1(S0);
-      Z[0] = fma2(c.nax, make_float2(S1 - S0, S2 - S1), X01);
-      Z[1] = fma2(c.nax, make_float2(S3 - S2, S4 - S3), X23);
-    } else {
-      Z[0] = X01;
-      Z[1] = X23;
-    }
-  }
+#include "step_kernel_body.cuh"
+#include "pair_node.cuh"
 
-  float2 o[2];
-  const float2 Bn[2] = {B0, B1};
-  if constexpr (ORDER == 2) {
-    float2 Ry[2], Sy[2], dSy[2];
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      Ry[m] = sub2(Bn[m], s.Fp[m]);
-      const float2 hy = mul2(c.q, add2(Ry[m], s.Ryp[m]));
-      if constexpr (SY > 0)
-        Sy[m] = make_float2(mc_half<LIM>(Ry[m].x, s.Ryp[m].x, hy.x),
-                            mc_half<LIM>(Ry[m].y, s.Ryp[m].y, hy.y));
-      else
-        Sy[m] = make_float2(mc_half<LIM>(s.Ryp[m].x, Ry[m].x, hy.x),
-                            mc_half<LIM>(s.Ryp[m].y, Ry[m].y, hy.y));
-      dSy[m] = sub2(Sy[m], s.Syp[m]);
-    }
-    // dS^y one column upwind in x
-    float2 dsu[2];
-    if constexpr (SX > 0) {
-      const float du = shfl_up1(dSy[1].y);
-      dsu[0] = make_float2(du, dSy[0].x);
-      dsu[1] = make_float2(dSy[0].y, dSy[1].x);
-    } else {
-      const float du = shfl_dn1(dSy[0].x);
-      dsu[0] = make_float2(dSy[0].y, dSy[1].x);
-      dsu[1] = make_float2(dSy[1].y, du);
-    }
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const float2 Zi = SY > 0 ? s.Z1[m] : s.Z2[m];
-      const float2 Zu = SY > 0 ? s.Z2[m] : s.Z1[m];
-      float2 v = fma2(c.cy, sub2(Zu, Zi), Zi);
-      v = fma2(c.by0, dSy[m], v);
-      o[m] = make_float2(fmaf(c.by1, dsu[m].x, v.x), fmaf(c.by1, dsu[m].y, v.y));
-      s.Ryp[m] = Ry[m];
-      s.Syp[m] = Sy[m];
-    }
-  } else {
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const float2 Zi = SY > 0 ? s.Z1[m] : s.Z2[m];
-      const float2 Zu = SY > 0 ? s.Z2[m] : s.Z1[m];
-      o[m] = fma2(c.cy, sub2(Zu, Zi), Zi);
-    }
-  }
-
-#pragma unroll
-  for (int m = 0; m < 2; ++m) {
-    if constexpr (SY > 0) {
-      out[2 * m] = s.pend[m].x;
-      out[2 * m + 1] = s.pend[m].y;
-      s.pend[m] = o[m];
-    } else {
-      out[2 * m] = o[m].x;
-      out[2 * m + 1] = o[m].y;
-    }
-    s.Fp[m] = Bn[m];
-    s.Z2[m] = s.Z1[m];
-    s.Z1[m] = Z[m];
-  }
+__device__ __forceinline__ void store_pair(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
+__device__ __forceinline__ void store_pair(__half* p, float2 v) {
+  *reinterpret_cast<__half2*>(p) = __floats2half2_rn(v.x, v.y);
 }
 
-// the advection state of the arithmetic type: FP32 packs column pairs
-template <typename T>
-struct AdvSel {
-  using State = AdvState<T>;
-};
-template <>
-struct AdvSel<float> {
-  using State = AdvState2;
-};
-
-#include "step_kernel_body.cuh"
+#include "step_stream.cuh"
 
 }  // namespace ctulbm

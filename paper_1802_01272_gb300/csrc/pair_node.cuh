@@ -1,0 +1,311 @@
+// pair_node.cuh -- the per-node part of the step (moments, force, collision)
+// for two x-neighbouring nodes at a time (included by lbm_kernels.cuh inside
+// namespace ctulbm).
+//
+// A value of both nodes is one V = PairOf<T>::type (float2 or double2).  In
+// FP32 every operation on whole pairs is one packed FP32x2 instruction
+// (sm_100+) and every shared-memory access of a pair one 8-byte access, so a
+// pair costs little more issue slots than a node does.
+
+// The constants of the collision phase as pairs.
+template <typename T>
+struct NodeConst {
+  using V = typename PairOf<T>::type;
+  V gw1, gw2, gw3, gw4, kw[6];
+  V om, ps, p00, p10, pg, p20, p30;
+  V lo, hi, nlo, nhi, lo2, hi2;
+  V w[3];
+  __device__ explicit NodeConst(const StepArgs<T>& P)
+      : gw1(dup2(P.gw1)), gw2(dup2(P.gw2)), gw3(dup2(P.gw3)), gw4(dup2(P.gw4)), om(dup2(P.omega)),
+        ps(dup2(P.ps)), p00(dup2(P.p00)), p10(dup2(P.p10)), pg(dup2(P.pg)), p20(dup2(P.p20)),
+        p30(dup2(P.p30)), lo(dup2(P.xlo)), hi(dup2(P.xhi)), nlo(dup2(-P.xlo)), nhi(dup2(-P.xhi)),
+        lo2(dup2(P.lo2)), hi2(dup2(P.hi2)) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) kw[i] = dup2(P.kw[i]);
+    w[0] = dup2(P.cls[0].w);
+    w[1] = dup2(P.cls[1].w);  // groups 1 and 2 share their weight
+    w[2] = dup2(P.cls[3].w);
+  }
+};
+
+// Rows of the moment rings around a pair: columns (c-2, c-1), (c, c+1), (c+2, c+3).
+template <typename V>
+struct Row6 {
+  V l, m, r;
+};
+template <typename T>
+__device__ __forceinline__ Row6<typename PairOf<T>::type> row6(const T* p) {
+  using V = typename PairOf<T>::type;
+  return {*reinterpret_cast<const V*>(p - 2), *reinterpret_cast<const V*>(p),
+          *reinterpret_cast<const V*>(p + 2)};
+}
+template <typename V>
+__device__ __forceinline__ Row6<V> add_rows(const Row6<V>& a, const Row6<V>& b) {
+  return {add2(a.l, b.l), add2(a.m, b.m), add2(a.r, b.r)};
+}
+template <typename V>
+__device__ __forceinline__ Row6<V> sub_rows(const Row6<V>& a, const Row6<V>& b) {
+  return {sub2(a.l, b.l), sub2(a.m, b.m), sub2(a.r, b.r)};
+}
+
+// dt g / ds at two nodes (Eq. eder) from the moment rings; ph[b + 2], dq[b + 2]
+// point at the pair's column in the ring row of lattice row + b, b = -2 .. 2.
+//  * grad(p^i - p^w): the fourth-order 5x5 gradient (4 D_h - D_2h)/3 of the
+//    isotropic 3x3 gradient D_h at spacings ds and 2 ds;
+//  * kappa grad(lap rho*): D_h of the isotropic 9-point Laplacian, the two
+//    composed into one 5x5 stencil on rho* - rho_ref (the Laplacian of a
+//    constant vanishes).
+// Both stencils are even across the derivative's direction, so rows are added
+// (for d/dx) or subtracted (for d/dy) first and the sums shared by the pair.
+template <typename T>
+__device__ __forceinline__ void pair_force(const NodeConst<T>& C, const T* const (&ph)[5],
+                                           const T* const (&dq)[5], typename PairOf<T>::type ir,
+                                           typename PairOf<T>::type& gx,
+                                           typename PairOf<T>::type& gy,
+                                           typename PairOf<T>::type& drho) {
+  using V = typename PairOf<T>::type;
+  using PO = PairOf<T>;
+  V px, py;
+  {
+    const Row6<V> t0 = row6(ph[2]), up = row6(ph[3]), dn = row6(ph[1]);
+    const Row6<V> t1 = add_rows(up, dn), d1 = sub_rows(up, dn);
+    const Row6<V> up2 = row6(ph[4]), dn2 = row6(ph[0]);
+    const Row6<V> d2 = sub_rows(up2, dn2);
+    const V t2l = add2(up2.l, dn2.l), t2r = add2(up2.r, dn2.r);
+    const V w1 = C.gw1, w2 = C.gw2, w3 = C.gw3, w4 = C.gw4;
+    const V al = fma2(w1, t0.l, mul2(w2, t1.l)), am = fma2(w1, t0.m, mul2(w2, t1.m)),
+            ar = fma2(w1, t0.r, mul2(w2, t1.r));
+    const V bl = fma2(w3, t0.l, mul2(w4, t2l)), br = fma2(w3, t0.r, mul2(w4, t2r));
+    px = sub2(PO::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
+    const V e1 = PO::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d2.r, d2.l);
+    py = sub2(fma2(w1, d1.m, mul2(w2, e1)), fma2(w3, d2.m, mul2(w4, e2)));
+  }
+  V lx, ly;
+  {
+    const Row6<V> t0 = row6(dq[2]), up = row6(dq[3]), dn = row6(dq[1]);
+    drho = t0.m;
+    const Row6<V> t1 = add_rows(up, dn), d1 = sub_rows(up, dn);
+    const Row6<V> up2 = row6(dq[4]), dn2 = row6(dq[0]);
+    const Row6<V> t2 = add_rows(up2, dn2), d2 = sub_rows(up2, dn2);
+    const V k0 = C.kw[0], k1 = C.kw[1], k2 = C.kw[2], k3 = C.kw[3], k4 = C.kw[4], k5 = C.kw[5];
+    const V al = fma2(k0, t0.l, fma2(k1, t1.l, mul2(k2, t2.l)));
+    const V am = fma2(k0, t0.m, fma2(k1, t1.m, mul2(k2, t2.m)));
+    const V ar = fma2(k0, t0.r, fma2(k1, t1.r, mul2(k2, t2.r)));
+    const V bl = fma2(k3, t0.l, fma2(k4, t1.l, mul2(k5, t2.l)));
+    const V br = fma2(k3, t0.r, fma2(k4, t1.r, mul2(k5, t2.r)));
+    lx = add2(PO::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
+    const V e1 = PO::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d1.r, d1.l);
+    const V h1 = PO::make(d2.m.y + d2.l.y, d2.r.x + d2.m.x), h2 = add2(d2.r, d2.l);
+    ly = fma2(k0, d1.m, fma2(k1, e1, fma2(k2, e2, fma2(k3, d2.m, fma2(k4, h1, mul2(k5, h2))))));
+  }
+  gx = fma2(ir, px, lx);
+  gy = fma2(ir, py, ly);
+}
+
+// Sums over the four sign patterns of each velocity group: d = sum f, sx and sy
+// = sums with the signs of xi_x and xi_y, t = with their product.
+template <typename V>
+struct GroupSums {
+  V d[4], sx[4], sy[4], t[4];
+};
+template <typename V, bool T_TOO, typename Load>
+__device__ __forceinline__ GroupSums<V> group_sums(Load f) {
+  GroupSums<V> g;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const V f0 = f(4 * m), f1 = f(4 * m + 1), f2 = f(4 * m + 2), f3 = f(4 * m + 3);
+    const V p = add2(f0, f2), q = add2(f1, f3), a = sub2(f0, f2), b = sub2(f1, f3);
+    g.d[m] = add2(p, q);
+    g.sx[m] = sub2(a, b);
+    g.sy[m] = add2(a, b);
+    if constexpr (T_TOO) g.t[m] = sub2(p, q);
+  }
+  return g;
+}
+
+// rho* - rho_ref, u* and p^i - p^w = rho T - [rho T/(1 - b rho) - a rho^2]
+// (Eqs. eder, evdw) of two nodes; f(k) loads velocity k of the pair.
+template <typename T, typename Load>
+__device__ __forceinline__ void pair_moments(const StepArgs<T>& P, Load f,
+                                             typename PairOf<T>::type& dr,
+                                             typename PairOf<T>::type& ux,
+                                             typename PairOf<T>::type& uy,
+                                             typename PairOf<T>::type& phi) {
+  using V = typename PairOf<T>::type;
+  const GroupSums<V> g = group_sums<V, false>(f);
+  dr = add2(g.d[0], add2(g.d[1], add2(g.d[2], g.d[3])));  // the heaviest group last
+  const V rho = add2(dup2(P.rho_ref), dr);
+  const V ir = PairOf<T>::make(rcp(rho.x), rcp(rho.y));
+  const V lo = dup2(P.xlo), hi = dup2(P.xhi);
+  ux = mul2(fma2(lo, add2(g.sx[0], g.sx[2]), mul2(hi, add2(g.sx[1], g.sx[3]))), ir);
+  uy = mul2(fma2(lo, add2(g.sy[0], g.sy[1]), mul2(hi, add2(g.sy[2], g.sy[3]))), ir);
+  const V rT = mul2(rho, dup2(P.Tt));
+  const V den = fma2(dup2(P.b), rho, dup2(T(-1)));  // -(1 - b rho)
+  const V q = PairOf<T>::make(rcp(den.x), rcp(den.y));
+  phi = fma2(mul2(dup2(P.a), rho), rho, fma2(rT, q, rT));
+}
+
+// The collision as a polynomial in the velocity components.  With x = xi_x,
+// y = xi_y, (u, v) = u*, (g, h) = dt g, w = dt/tau, s = (T - 1)/2:
+//   [w f^eq + dt F_k - w w_k rho_ref] / (w_k rho)
+//     = sum_{m+n<=3} c_mn x^m y^n
+// (Eqs. herfeq, herforce: xi.u = x u + y v and xi.g = x g + y h expanded), and
+// f^{n+1} = (1 - w) f* + w_k rho sum c_mn x^m y^n.  The velocities are the
+// products of x, y in {+-lo, +-hi}, so the polynomial is evaluated by its even
+// and odd parts in y, then in x: 50 operations for the 16 values (the form in
+// xi.u and xi.g of each velocity takes 112).
+template <typename V>
+struct Poly {
+  V c00, c10, c01, c20, c11, c02, c30, c21, c12, c03;
+};
+
+template <typename T>
+__device__ __forceinline__ Poly<typename PairOf<T>::type> collision_poly(
+    const NodeConst<T>& C, typename PairOf<T>::type drho, typename PairOf<T>::type ir,
+    typename PairOf<T>::type u, typename PairOf<T>::type v, typename PairOf<T>::type g,
+    typename PairOf<T>::type h) {
+  using V = typename PairOf<T>::type;
+  const V om = C.om, s = C.ps;
+  const V a = fma2(om, u, g), b = fma2(om, v, h);  // w u + dt g
+  const V hu = mul2(mul2(dup2(T(0.5)), u), u), hv = mul2(mul2(dup2(T(0.5)), v), v), uv = mul2(u, v);
+  const V k = add2(hu, hv);                 // u^2 / 2
+  const V gu = fma2(g, u, mul2(h, v));      // dt g.u
+  const V su = add2(s, hu), sv = add2(s, hv);
+  Poly<V> p;
+  p.c00 = sub2(fma2(om, sub2(mul2(drho, ir), k), C.p00), gu);
+  const V K = sub2(sub2(C.p10, mul2(om, k)), gu), G = sub2(C.pg, k);
+  p.c10 = fma2(K, u, mul2(G, g));
+  p.c01 = fma2(K, v, mul2(G, h));
+  p.c20 = fma2(om, hu, fma2(u, g, C.p20));
+  p.c02 = fma2(om, hv, fma2(v, h, C.p20));
+  p.c11 = fma2(v, a, mul2(u, h));
+  p.c30 = fma2(C.p30, mul2(hu, u), mul2(a, su));
+  p.c03 = fma2(C.p30, mul2(hv, v), mul2(b, sv));
+  p.c21 = fma2(b, su, mul2(g, uv));
+  p.c12 = fma2(a, sv, mul2(h, uv));
+  return p;
+}
+
+// Calls put(k, value) with the polynomial's value at velocity k, k = 0 .. 15.
+template <typename T, typename V, typename Put>
+__device__ __forceinline__ void poly_each(const NodeConst<T>& C, const Poly<V>& p, Put put) {
+#pragma unroll
+  for (int iy = 0; iy < 2; ++iy) {
+    const V y = iy ? C.hi : C.lo, ny = iy ? C.nhi : C.nlo, y2 = iy ? C.hi2 : C.lo2;
+    const V e0 = fma2(p.c02, y2, p.c00), o0 = fma2(p.c03, y2, p.c01), e1 = fma2(p.c12, y2, p.c10);
+#pragma unroll
+    for (int sy = 0; sy < 2; ++sy) {
+      const V yy = sy ? ny : y;
+      const V a0 = fma2(yy, o0, e0), a1 = fma2(yy, p.c11, e1), a2 = fma2(yy, p.c21, p.c20);
+#pragma unroll
+      for (int ix = 0; ix < 2; ++ix) {
+        const V x = ix ? C.hi : C.lo, nx = ix ? C.nhi : C.nlo, x2 = ix ? C.hi2 : C.lo2;
+        const V e = fma2(a2, x2, a0), o = fma2(p.c30, x2, a1);
+        const int k = 4 * (2 * iy + ix);  // signs in a group: (+,+), (-,+), (-,-), (+,-)
+        put(k + (sy ? 3 : 0), fma2(x, o, e));
+        put(k + (sy ? 2 : 1), fma2(nx, o, e));
+      }
+    }
+  }
+}
+
+// Eq. (ereg) inside the collision: f* is replaced by f^eq + w [H2:A2/2 + H3:A3/6],
+// A_n = sum f^neq xi^n, which is a polynomial in (x, y) as well; it joins the
+// collision's with the factor 1 - w, and f^{n+1} = w_k * (the sum) needs f*
+// only through its second and third moments.  p comes in as collision_poly's
+// and leaves as the polynomial of f^{n+1} / w_k (s1 = 1 - w, rw = rho, see pair_collide).
+template <typename T, typename Load>
+__device__ __forceinline__ void regularised_poly(const StepArgs<T>& P, Load f,
+                                                 Poly<typename PairOf<T>::type>& p,
+                                                 typename PairOf<T>::type drho,
+                                                 typename PairOf<T>::type rho,
+                                                 typename PairOf<T>::type u,
+                                                 typename PairOf<T>::type v,
+                                                 typename PairOf<T>::type s1,
+                                                 typename PairOf<T>::type rw) {
+  using V = typename PairOf<T>::type;
+  const GroupSums<V> q = group_sums<V, true>(f);
+  const T lo = P.xlo, hi = P.xhi, l2 = P.lo2, h2 = P.hi2;
+  auto comb = [&](T a, V x, T b, V y) { return fma2(dup2(a), x, mul2(dup2(b), y)); };
+  const V mxx = comb(l2, add2(q.d[0], q.d[2]), h2, add2(q.d[1], q.d[3]));
+  const V myy = comb(l2, add2(q.d[0], q.d[1]), h2, add2(q.d[2], q.d[3]));
+  const V mxy = fma2(dup2(lo * hi), add2(q.t[1], q.t[2]), comb(l2, q.t[0], h2, q.t[3]));
+  const V mxxx = comb(lo * l2, add2(q.sx[0], q.sx[2]), hi * h2, add2(q.sx[1], q.sx[3]));
+  const V myyy = comb(lo * l2, add2(q.sy[0], q.sy[1]), hi * h2, add2(q.sy[2], q.sy[3]));
+  const V mxxy = add2(comb(lo * l2, q.sy[0], hi * h2, q.sy[3]), comb(lo * h2, q.sy[1], hi * l2, q.sy[2]));
+  const V mxyy = add2(comb(lo * l2, q.sx[0], hi * h2, q.sx[3]), comb(hi * l2, q.sx[1], lo * h2, q.sx[2]));
+  const V Tt = dup2(P.Tt), ref = dup2(P.rho_ref), half = dup2(T(0.5)), sixth = dup2(T(1) / T(6));
+  const V uu = mul2(u, u), vv = mul2(v, v), uv = mul2(u, v);
+  const V Axx = sub2(add2(mxx, ref), mul2(rho, add2(uu, Tt)));
+  const V Ayy = sub2(add2(myy, ref), mul2(rho, add2(vv, Tt)));
+  const V Axy = sub2(mxy, mul2(rho, uv));
+  const V T3 = dup2(T(3) * P.Tt);
+  const V ru = mul2(rho, u), rv = mul2(rho, v);
+  const V Axxx = sub2(mxxx, mul2(ru, add2(uu, T3))), Ayyy = sub2(myyy, mul2(rv, add2(vv, T3)));
+  const V Axxy = sub2(mxxy, mul2(rv, add2(uu, Tt))), Axyy = sub2(mxyy, mul2(ru, add2(vv, Tt)));
+  // f^eq / w - rho_ref = drho + rho (P - 1), P - 1 in powers of x, y
+  const V s = dup2(P.ps), hu = mul2(half, uu), hv = mul2(half, vv);
+  const V k = add2(hu, hv), su = add2(hu, s), sv = add2(hv, s);
+  const V q10 = sub2(dup2(T(1) - T(4) * P.ps), k);
+  const V third = dup2(T(1) / T(3));
+  Poly<V> r;
+  r.c00 = sub2(sub2(drho, mul2(rho, add2(k, dup2(T(2) * P.ps)))), mul2(half, add2(Axx, Ayy)));
+  r.c10 = sub2(mul2(ru, q10), mul2(half, add2(Axxx, Axyy)));
+  r.c01 = sub2(mul2(rv, q10), mul2(half, add2(Ayyy, Axxy)));
+  r.c20 = fma2(rho, su, mul2(half, Axx));
+  r.c02 = fma2(rho, sv, mul2(half, Ayy));
+  r.c11 = fma2(rho, uv, Axy);
+  r.c30 = fma2(ru, fma2(third, hu, s), mul2(sixth, Axxx));
+  r.c03 = fma2(rv, fma2(third, hv, s), mul2(sixth, Ayyy));
+  r.c21 = fma2(rv, su, mul2(half, Axxy));
+  r.c12 = fma2(ru, sv, mul2(half, Axyy));
+  auto join = [&](V& c, V d) { c = fma2(s1, d, mul2(rw, c)); };
+  join(p.c00, r.c00);
+  join(p.c10, r.c10);
+  join(p.c01, r.c01);
+  join(p.c20, r.c20);
+  join(p.c11, r.c11);
+  join(p.c02, r.c02);
+  join(p.c30, r.c30);
+  join(p.c21, r.c21);
+  join(p.c12, r.c12);
+  join(p.c03, r.c03);
+}
+
+// Collision of two nodes: f(k) loads f*_k, put(k, value) receives f^{n+1}_k.
+// The density reservoir (Sec. III A) multiplies the result by s: the stored
+// deviation becomes s f' + w rho_ref (s - 1), which is the same expression with
+// the factors s1 = s (1 - w) and rw = s rho and a constant term: cr = rho_ref
+// (s - 1) / rw (rw = rho_ext to rounding), or rho_ref (s - 1) itself for the
+// regularised collision.
+template <typename T, bool REGU, typename Load, typename Put>
+__device__ __forceinline__ void pair_collide(const StepArgs<T>& P, const NodeConst<T>& C, Load f,
+                                             Put put,
+                                             typename PairOf<T>::type drho,
+                                             typename PairOf<T>::type rho,
+                                             typename PairOf<T>::type ir,
+                                             typename PairOf<T>::type u,
+                                             typename PairOf<T>::type v,
+                                             typename PairOf<T>::type g,
+                                             typename PairOf<T>::type h,
+                                             typename PairOf<T>::type s1,
+                                             typename PairOf<T>::type rw,
+                                             typename PairOf<T>::type cr) {
+  using V = typename PairOf<T>::type;
+  Poly<V> p = collision_poly<T>(C, drho, ir, u, v, g, h);
+  if constexpr (REGU) {
+    regularised_poly<T>(P, f, p, drho, rho, u, v, s1, rw);
+    p.c00 = add2(p.c00, cr);
+    poly_each(C, p, [&](int k, V q) {
+      const int grp = k >> 2;
+      put(k, mul2(C.w[grp == 0 ? 0 : (grp == 3 ? 2 : 1)], q));
+    });
+  } else {
+    p.c00 = add2(p.c00, cr);
+    const V sw[3] = {mul2(C.w[0], rw), mul2(C.w[1], rw), mul2(C.w[2], rw)};
+    poly_each(C, p, [&](int k, V q) {
+      const int grp = k >> 2;
+      put(k, fma2(s1, f(k), mul2(sw[grp == 0 ? 0 : (grp == 3 ? 2 : 1)], q)));
+    });
+  }
+}

@@ -26,7 +26,7 @@ int step_occupancy_f32(int order, int lim, bool vec, bool regu, size_t smem) {
 namespace {
 template <int ORDER, int LIM, bool REGU>
 void* batch_ptr() {
-  return reinterpret_cast<void*>(&step_batch_kernel<float, ORDER, LIM, true, REGU>);
+  return reinterpret_cast<void*>(&stream_batch_kernel<ORDER, LIM, REGU>);
 }
 template <bool REGU>
 void* batch_by_scheme(int order, int lim) {
@@ -62,6 +62,7 @@ int step_batch_occupancy_f32(int order, int lim, bool regu, size_t smem) {
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return 0;
+  if (!stream_regs_ok(fn)) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, NT, smem) != cudaSuccess) return 0;
   return n;

@@ -307,28 +307,17 @@ __device__ __forceinline__ void seam_fixup(const StepArgs<T>& P, const Smem<T, S
 // P1 for one warp quadrant: the RPI staged rows of the batch in slot `sbase`,
 // advected rows to the f* ring at `fbase` (thread's plane and group).
 template <int SX, int SY, int ORDER, int LIM, typename T, typename ST>
-__device__ __forceinline__ void advect_batch(typename AdvSel<T>::State& st, const VelConst<T>& vc,
+__device__ __forceinline__ void advect_batch(AdvState<T>& st, const VelConst<T>& vc,
                                              const ST* sbase, T* fa, T* fb) {
   // rows 0, 1 of the batch go to ring rows fa, fa + FRS; rows 2, 3 to fb, fb + FRS
   constexpr int SCOL = scol_of<ST>();
-  if constexpr (sizeof(T) == 4) {
-    const VelPairs vp = vel_pairs<SX>(vc);
 #pragma unroll
-    for (int r = 0; r < RPI; ++r) {
-      float out[4];
-      advect_row2<SX, SY, ORDER, LIM>(st, sbase + r * (16 * SCOL), vp, out);
-      *reinterpret_cast<float4*>((r < 2 ? fa : fb) + (r & 1) * FRS) =
-          make_float4(out[0], out[1], out[2], out[3]);
-    }
-  } else {
-#pragma unroll
-    for (int r = 0; r < RPI; ++r) {
-      T out[4];
-      advect_row<SX, SY, ORDER, LIM>(st, sbase + r * (16 * SCOL), vc, out);
-      T* dst = (r < 2 ? fa : fb) + (r & 1) * FRS;
-      reinterpret_cast<double2*>(dst)[0] = make_double2(out[0], out[1]);
-      reinterpret_cast<double2*>(dst)[1] = make_double2(out[2], out[3]);
-    }
+  for (int r = 0; r < RPI; ++r) {
+    T out[4];
+    advect_row<SX, SY, ORDER, LIM>(st, sbase + r * (16 * SCOL), vc, out);
+    T* dst = (r < 2 ? fa : fb) + (r & 1) * FRS;
+    reinterpret_cast<double2*>(dst)[0] = make_double2(out[0], out[1]);
+    reinterpret_cast<double2*>(dst)[1] = make_double2(out[2], out[3]);
   }
 }
 
@@ -402,7 +391,7 @@ __device__ __forceinline__ void run_segment(const StepArgs<T>& P, const Smem<T, 
   if (VEC && P.tma_out && tid == PRODUCER) bulk_wait_read<0>();
   __syncthreads();  // previous segment done with the rings and the slots
 
-  typename AdvSel<T>::State st;
+  AdvState<T> st;
   memset(&st, 0, sizeof(st));
 
   constexpr int SCOL = Smem<T, ST>::SCOL;
@@ -847,31 +836,3 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 1)
   retire_cta(P.sched);
 }
 
-// Several lattices advanced by one launch: their work items are concatenated
-// and claimed from one counter; each lattice brings its own tensor maps.
-template <typename T, int ORDER, int LIM, bool VEC, bool REGU>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 1)
-    step_batch_kernel(const __grid_constant__ BatchArgs<T> B) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const Smem<T, T> S(smem_raw);
-  __shared__ long long s_item;
-  init_cta_barriers(S.dsums, S.bar, S.abort);
-  int i = 0;
-  unsigned gb = 0, gi = 0;
-  double dmass = 0.0;  // unused: batched launches carry no fused diagnostics
-  for (;;) {
-    const long long item = claim_item(B.sched, &s_item);
-    if (item >= B.item_start[B.count]) break;
-    while (B.item_start[i + 1] <= item) ++i;
-    const StepArgs<T>& P = B.L[i];
-    const long long local = item - B.item_start[i];
-    int strip;
-    long long rb;
-    item_coords(local, P.nstrip, P.items / P.nstrip, strip, rb);
-    const int ys = (int)(rb * P.row_block);
-    const int ye = min(P.Ly, ys + P.row_block);
-    run_segment<T, T, ORDER, LIM, VEC, false, REGU>(P, S, strip, ys, ye, B.maps[i].m, gb, gi, dmass);
-  }
-  drain_copies(S, gi);
-  retire_cta(B.sched);
-}

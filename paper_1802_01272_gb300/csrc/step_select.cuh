@@ -6,11 +6,20 @@
 // plain step's loop carries no code for the others.
 #pragma once
 
+// The stream kernel's roles trade registers, which must add up (see STREAM_REGS).
+inline bool stream_regs_ok(const void* fn) {
+  cudaFuncAttributes a;
+  return cudaFuncGetAttributes(&a, fn) == cudaSuccess && a.numRegs == STREAM_REGS;
+}
+
 template <typename T, typename ST>
 struct StepSelect {
   template <int ORDER, int LIM, bool VEC, bool DIAG, bool REGU>
   static void* ptr() {
-    return reinterpret_cast<void*>(&step_kernel<T, ST, ORDER, LIM, VEC, DIAG, REGU>);
+    if constexpr (sizeof(T) == 4)
+      return reinterpret_cast<void*>(&stream_kernel<ST, ORDER, LIM, VEC, DIAG, REGU>);
+    else
+      return reinterpret_cast<void*>(&step_kernel<T, ST, ORDER, LIM, VEC, DIAG, REGU>);
   }
   template <bool VEC, bool DIAG, bool REGU>
   static void* by_scheme(int order, int lim) {
@@ -43,6 +52,7 @@ struct StepSelect {
     int occ = 1 << 30;
     for (int d = 0; d < 2; ++d) {
       void* fn = select(order, lim, vec, d == 1, regu);
+      if (sizeof(T) == 4 && !stream_regs_ok(fn)) return 0;
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess)
         return 0;
