@@ -99,7 +99,7 @@ def load_peaks():
     return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("lbm_kernels.cuh", "pair_node.cuh", "step_stream.cuh", "step_kernel_body.cuh",
+KERNEL_SOURCES = ("lbm_kernels.cuh", "pair_node.cuh", "step_stream.cuh", "step_split64.cuh",
                   "step_select.cuh", "step_fp32.cu", "step_fp64.cu", "step_fp16.cu")
 
 

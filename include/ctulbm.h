@@ -144,7 +144,7 @@ int lbm_set_f_device(lbm_handle* h, const double* f);
 int lbm_get_f_device(lbm_handle* h, double* f);
 
 /* Advance n >= 0 steps on the handle's stream (asynchronous; one fused kernel
- * per step).  From 32 steps on, whole blocks of 16 steps go out as one CUDA
+ * per step, in FP64 an advection and a collision kernel).  From 32 steps on, whole blocks of 16 steps go out as one CUDA
  * graph launch (built on first use per handle; the same kernels, in order). */
 int lbm_step(lbm_handle* h, int64_t n);
 
@@ -288,6 +288,7 @@ int lbm_batch_get_info(lbm_batch* b, lbm_batch_info* out);
 /* Launch geometry of the handle's fused step kernel (no counterpart in the
  * paper: for tuning, benchmarking and tests).
  *   grid          CTAs of the persistent launch (SMs x resident CTAs at most)
+ *                 (FP64: of the advection kernel, as the next two)
  *   threads       threads per CTA
  *   smem_bytes    dynamic shared memory per CTA
  *   strips        strips of 56 output columns across x

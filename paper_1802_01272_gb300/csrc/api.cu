@@ -26,7 +26,6 @@ struct lbm_handle {
   void* f[2] = {nullptr, nullptr};
   int cur = 0;
   unsigned int* d_err = nullptr;
-  unsigned long long* d_sched = nullptr;  // work-item counters of the step kernel
   DiagAcc* d_acc = nullptr;
   double* d_work = nullptr;       // 3 planes of FP64 for moments / init staging
   size_t work_elems = 0;
@@ -93,26 +92,19 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// f [16][Ly][Lx] as a 3-D tensor ordered (x, plane, row), read in boxes of
-// `cols` columns x 16 planes x `rows` rows: a box is [rows][16][cols] in
-// shared memory (consecutive rows of the staging ring).  False when the
-// encoder is unavailable or rejects the layout (the kernel then stages every
-// strip by per-thread copies).
-bool encode_row_map(void* base, size_t elem, int Lx, int Ly, int cols, int rows,
-                    CUtensorMap* out) {
+// FP64 f [16][Ly][Lx] as a 3-D tensor ordered (x, plane, row), read in boxes of
+// `cols` columns x 1 plane x `rows` rows.  False when the encoder is unavailable or
+// rejects the layout (the kernels then load value by value).
+bool encode_plane_map(void* base, int Lx, int Ly, int cols, int rows, CUtensorMap* out) {
   const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc || Lx < cols || Ly < rows) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)Lx, 16, (cuuint64_t)Ly};
-  const cuuint64_t strides[2] = {(cuuint64_t)Lx * (cuuint64_t)Ly * elem, (cuuint64_t)Lx * elem};
-  const cuuint32_t box[3] = {(cuuint32_t)cols, 16, (cuuint32_t)rows};
+  const cuuint64_t strides[2] = {(cuuint64_t)Lx * (cuuint64_t)Ly * 8, (cuuint64_t)Lx * 8};
+  const cuuint32_t box[3] = {(cuuint32_t)cols, 1, (cuuint32_t)rows};
   const cuuint32_t estr[3] = {1, 1, 1};
-  const CUtensorMapDataType type = elem == 8   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64
-                                   : elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                               : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  return enc(out, type, 3,
-             base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return enc(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, base, dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // The same for the stream kernel, whose advect warps each stage the four planes
@@ -130,25 +122,6 @@ bool encode_quadrant_map(void* base, size_t elem, int Lx, int Ly, int cols, int 
   const CUtensorMapDataType type =
       elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   return enc(out, type, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// f [16][Ly][Lx] as a 3-D tensor ordered (x, row, plane), written in tiles of
-// TW columns x RPI rows x 16 planes: a tile is [16][RPI][TW] in shared memory
-// (the collision's plane-major output tile).  False when the encoder is
-// unavailable or rejects the layout (the kernel then stores per thread).
-bool encode_tile_map(void* base, size_t elem, int Lx, int Ly, CUtensorMap* out) {
-  const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc || Lx < TW || Ly < RPI) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)Lx, (cuuint64_t)Ly, 16};
-  const cuuint64_t strides[2] = {(cuuint64_t)Lx * elem, (cuuint64_t)Lx * (cuuint64_t)Ly * elem};
-  const cuuint32_t box[3] = {(cuuint32_t)TW, (cuuint32_t)RPI, 16};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUtensorMapDataType type = elem == 8   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64
-                                   : elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                               : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  return enc(out, type, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -185,7 +158,6 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   a.nstrip = h->nstrip;
   a.row_block = h->row_block;
   a.items = (long long)((p.Ly + h->row_block - 1) / h->row_block) * h->nstrip;
-  a.sched = h->d_sched;
   a.diag_mass = nullptr;
   a.diag_sums = nullptr;
   a.diag_thr = (T)0;
@@ -214,8 +186,6 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   }
   a.omega = (T)om;
   a.one_m_omega = (T)(1.0 - om);
-  a.om2 = (T)(0.5 * om);
-  a.om6 = (T)(om / 6.0);
   a.rho_ext = (T)p.rho_ext;
   a.irho_ext = (T)(p.rho_ext != 0.0 ? 1.0 / p.rho_ext : 0.0);
   const int Lmin = p.Lx < p.Ly ? p.Lx : p.Ly;
@@ -235,16 +205,7 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   a.pg = (T)(3.0 - 2.0 * p.T);
   a.p20 = (T)(om * ps);
   a.p30 = (T)(-2.0 * om / 3.0);
-  for (int grp = 0; grp < 4; ++grp) {
-    const int k = 4 * grp;
-    const double x2 = h->xi[k][0] * h->xi[k][0] + h->xi[k][1] * h->xi[k][1];
-    const double Ak = (p.T - 1.0) * (x2 - 2.0) / 2.0, Bk = (p.T - 1.0) * (x2 - 4.0) / 2.0;
-    a.cls[grp].omA = (T)(om * Ak);
-    a.cls[grp].Ak = (T)Ak;
-    a.cls[grp].omB = (T)(om * Bk);
-    a.cls[grp].Bk = (T)Bk;
-    a.cls[grp].w = (T)h->w[k];
-  }
+  for (int i = 0; i < 3; ++i) a.w[i] = (T)h->w[4 * i + (i == 2 ? 4 : 0)];
   double gb[16], gt[16];
   const double uw = p.shear_rate * p.Ly * p.ds / 2.0;
   feq_host(p, h->xi, h->w, p.rho_ext, -uw, 0.0, gb);
@@ -253,36 +214,24 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
     const double x = h->xi[k][0], y = h->xi[k][1];
     const double ax = std::fabs(x), ay = std::fabs(y);
     const double cx = lam * ax, cy = lam * ay;
-    const double hx = 0.5 * ax * (1.0 - cx), hy = 0.5 * ay * (1.0 - cy);
-    const double x2 = x * x + y * y;
-    const double Ak = (p.T - 1.0) * (x2 - 2.0) / 2.0, Bk = (p.T - 1.0) * (x2 - 4.0) / 2.0;
+    const double hx = 0.5 * ax * (1.0 - cx);
     VelConst<T>& v = a.v[k];
     v.xi_x = (T)x;
     v.xi_y = (T)y;
     v.w = (T)h->w[k];
     // CTU2 per node (Sec. II C 2 collected): with Z(j) = f - c_x (f - f(i - s_x))
     // - 2 lam hx dS^x(j), the update is Z(j) + c_y (Z(j - s_y) - Z(j))
-    // - 2 lam hy [(1 - c_x) dS^y(i) + c_x dS^y(i - s_x)] on the kernel's
-    // half-limited jumps (hence the factors 2).  The interpolations
-    // f + c (g - f) return f exactly for g = f, so the CTU1 weights of a
-    // uniform state sum to 1 in any precision.
+    // - 2 lam hy [(1 - c_x) dS^y(i) + c_x dS^y(i - s_x)] on the kernels'
+    // half-limited jumps (hence the factors 2); 2 lam hy = c_y (1 - c_y).  The
+    // interpolations f + c (g - f) return f exactly for g = f, so the CTU1 weights
+    // of a uniform state sum to 1 in any precision.
     v.cx = (T)cx;
     v.cy = (T)cy;
     v.ax = (T)(2.0 * lam * hx);
-    v.by0 = (T)(-2.0 * lam * hy * (1.0 - cx));
-    v.by1 = (T)(-2.0 * lam * hy * cx);
     v.qy0 = (T)((1.0 - cy) * (1.0 - cx));
     v.qy1 = (T)((1.0 - cy) * cx);
     v.gbot = (T)(gb[k] - h->w[k] * rr);
     v.gtop = (T)(gt[k] - h->w[k] * rr);
-    // Eq. (ereg): w [ H2:A2 / 2! + H3:A3 / 3! ] over the independent components
-    v.r2xx = (T)(0.5 * (x * x - 1.0));
-    v.r2xy = (T)(x * y);
-    v.r2yy = (T)(0.5 * (y * y - 1.0));
-    v.r3xxx = (T)((x * x * x - 3.0 * x) / 6.0);
-    v.r3xxy = (T)(0.5 * (x * x * y - y));
-    v.r3xyy = (T)(0.5 * (x * y * y - x));
-    v.r3yyy = (T)((y * y * y - 3.0 * y) / 6.0);
   }
 }
 
@@ -373,6 +322,65 @@ long long pick_row_block(int Ly, int nstrip, long long grid) {
   return best;
 }
 
+// The FP64 advection hands out warp tasks: a plane of half a strip (32 per strip) by
+// a part of a row block.  An SM's FP64 pipe takes a warp instruction every 16 cycles,
+// one warp gives it one every ~170: a row of n tasks on an SM costs max(16 n, 170),
+// and a task of r rows r + 1 of them.  The split that minimises that for the busiest
+// SM (128^2 at 16-row blocks, parts of 16 and 8 rows: 15.7 and 9.1 us).
+double cost_f64(long long tasks, long long nsm, long long rows) {
+  const double n = (double)((tasks + nsm - 1) / nsm);
+  return (16.0 * n > 170.0 ? 16.0 * n : 170.0) * (double)(rows + 1);
+}
+int pick_sub_f64(int Ly, int nstrip, int rb, long long nsm) {
+  int best = 1;
+  double cost = 0.0;
+  for (int sub = 1; sub <= 8 && sub <= rb; ++sub) {
+    const int rows = (rb + sub - 1) / sub;
+    const double c = cost_f64((long long)((Ly + rb - 1) / rb) * nstrip * 32 * sub, nsm, rows);
+    if (sub == 1 || c < cost) {
+      cost = c;
+      best = sub;
+    }
+  }
+  return best;
+}
+long long pick_row_block_f64(int Ly, int nstrip, long long nsm) {
+  long long best = 16;
+  double cost = 0.0;
+  for (int rb = 16; rb <= 256; rb += 4) {
+    const int sub = pick_sub_f64(Ly, nstrip, rb, nsm);
+    const double c = cost_f64((long long)((Ly + rb - 1) / rb) * nstrip * 32 * sub, nsm,
+                              (rb + sub - 1) / sub);
+    if (cost == 0.0 || c < cost) {
+      cost = c;
+      best = rb;
+    }
+    if (rb >= Ly) break;
+  }
+  return best;
+}
+
+int scheme_limiter(const lbm_handle* h) { return h->p.ctu_order == 1 ? 0 : h->p.limiter; }
+
+// Resident CTAs per SM of the handle's step kernel (FP64: of the advection); 0 on error.
+int occupancy(const lbm_handle* h) {
+  const int o = h->p.ctu_order, lim = scheme_limiter(h);
+  const bool regu = h->p.regularize != 0;
+  return h->elem == 4   ? step_occupancy_f32(o, lim, h->vec, regu, h->smem)
+         : h->elem == 2 ? step_occupancy_f16(o, lim, h->vec, regu, h->smem)
+                        : step_occupancy_f64(o, lim);
+}
+
+// CTAs of a launch with row blocks of rb rows, at most ctas per SM: one per item, in
+// FP64 as many on every SM as its share of the warp tasks fills (they are dealt out
+// CTA by CTA).
+int grid_for(const lbm_handle* h, long long rb, int nsm, int ctas) {
+  const long long items = (h->p.Ly + rb - 1) / rb * h->nstrip, gmax = (long long)nsm * ctas;
+  const long long per = 8LL * nsm, tasks = 32LL * h->a64.sub * items;
+  const long long want = h->elem == 8 ? (tasks + per - 1) / per * nsm : items;
+  return (int)(want < gmax ? want : gmax);
+}
+
 int check_device_error(lbm_handle* h) {
   unsigned int e = 0;
   if (cudaMemcpyAsync(&e, h->d_err, sizeof(e), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
@@ -434,26 +442,20 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
   if ((e = cudaMalloc(&h->f[0], bytes)) != cudaSuccess ||
       (e = cudaMalloc(&h->f[1], bytes)) != cudaSuccess ||
       (e = cudaMalloc(&h->d_err, sizeof(unsigned int))) != cudaSuccess ||
-      (e = cudaMalloc(&h->d_acc, sizeof(DiagAcc))) != cudaSuccess ||
-      (e = cudaMalloc(&h->d_sched, 2 * sizeof(unsigned long long))) != cudaSuccess) {
+      (e = cudaMalloc(&h->d_acc, sizeof(DiagAcc))) != cudaSuccess) {
     lbm_destroy(h);
     return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
   }
   cudaMemsetAsync(h->d_err, 0, sizeof(unsigned int), h->stream);
-  cudaMemsetAsync(h->d_sched, 0, 2 * sizeof(unsigned long long), h->stream);
 
-  // tensor maps: rows of f^n staged by tensor copies (row strides and the
-  // staging window's start must be 16-byte multiples: Lx a multiple of 4
-  // values, 8 for half), output tiles stored by tensor stores
+  // tensor maps: rows of f^n staged by tensor copies (row strides and a staging
+  // window's start must be 16-byte multiples: Lx a multiple of 4 values, 8 for half)
   std::memset(h->tmap, 0, sizeof(h->tmap));
-  bool tin = (p->Lx % (h->elem == 2 ? 8 : 4)) == 0, tout = tin;
-  tin = tin && p->Lx >= (h->elem == 2 ? 72 : 68);
+  bool tin = (p->Lx % (h->elem == 2 ? 8 : 4)) == 0 && p->Lx >= (h->elem == 2 ? 72 : 68);
   const int last = (p->Lx - 1) / TW;  // the last strip
   for (int i = 0; i < 2; ++i) {
     if (h->elem == 8) {
-      tin = tin && encode_row_map(h->f[i], 8, p->Lx, p->Ly, scol_of<double>(), RPI, &h->tmap[i].m[0]) &&
-            encode_row_map(h->f[i], 8, p->Lx, p->Ly, scol_of<double>(), 1, &h->tmap[i].m[1]);
-      tout = tout && encode_tile_map(h->f[1 - i], 8, p->Lx, p->Ly, &h->tmap[i].m[2]);
+      tin = tin && encode_plane_map(h->f[i], p->Lx, p->Ly, step64_cols(), RPI, &h->tmap[i].m[0]);
     } else {
       // columns of a strip's staging, and of the runs at the left and right seam
       const int soff = h->elem == 2 ? StreamLayout<__half>::SOFF : StreamLayout<float>::SOFF;
@@ -464,35 +466,28 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
                       encode_quadrant_map(h->f[i], h->elem, p->Lx, p->Ly, cols[m], SR, &h->tmap[i].m[m]));
     }
   }
-  tin = tout = tin && tout;
-  h->vec = tin;  // else every strip stages by per-thread loads
+  h->vec = tin;  // else every strip is staged value by value
 
   // launch geometry: strips of TW output columns, rows split evenly over a
   // persistent grid of (SMs x resident CTAs), at least 48 rows per CTA
   h->nstrip = (p->Lx + TW - 1) / TW;
-  h->smem = step_smem_bytes(h->elem, h->elem == 8 ? 8 : 4);
-  const int lim = p->ctu_order == 1 ? 0 : p->limiter;
-  const bool regu = p->regularize != 0;
-  int occ = h->elem == 4   ? step_occupancy_f32(p->ctu_order, lim, h->vec, regu, h->smem)
-            : h->elem == 2 ? step_occupancy_f16(p->ctu_order, lim, h->vec, regu, h->smem)
-                           : step_occupancy_f64(p->ctu_order, lim, h->vec, regu, h->smem);
+  h->smem = h->elem == 8 ? 0 : step_smem_bytes(h->elem);
+  const int occ = occupancy(h);
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
   if (occ < 1 || nsm < 1) {
     lbm_destroy(h);
     return LBM_ERR_CUDA;
   }
-  const long long grid_max = (long long)nsm * occ;
-  const long long rb = pick_row_block(p->Ly, h->nstrip, grid_max);
-  h->row_block = (int)rb;
-  const long long items = (long long)((p->Ly + rb - 1) / rb) * h->nstrip;
-  h->grid = (int)(items < grid_max ? items : grid_max);
+  h->row_block = (int)(h->elem == 8 ? pick_row_block_f64(p->Ly, h->nstrip, nsm)
+                                    : pick_row_block(p->Ly, h->nstrip, (long long)nsm * occ));
+  h->a64.sub = pick_sub_f64(p->Ly, h->nstrip, h->row_block, nsm);
+  h->grid = grid_for(h, h->row_block, nsm, occ);
   if (h->elem == 8)
     fill_step_args<double>(h, h->a64);
   else
     fill_step_args<float>(h, h->a32);
   h->a32.tma_in = h->a64.tma_in = tin;
-  h->a32.tma_out = h->a64.tma_out = tout;
   AuxArgs& x = h->aux;
   x.Lx = p->Lx;
   x.Ly = p->Ly;
@@ -520,7 +515,6 @@ void lbm_destroy(lbm_handle* h) {
   cudaFree(h->f[1]);
   cudaFree(h->d_err);
   cudaFree(h->d_acc);
-  cudaFree(h->d_sched);
   cudaFree(h->d_work);
   delete h;
 }
@@ -613,18 +607,36 @@ namespace {
 
 constexpr int GRAPH_STEPS = 16;  // steps per graph launch (even: the buffers come back)
 
-// One step launch from f[c] to f[1 - c].
+// One step launch: from f[c] to f[1 - c]; in FP64 from f[c] back to f[c], with the
+// advected f in f[1 - c].
 cudaError_t launch_one(lbm_handle* h, int c, int lim) {
-  if (h->elem != 8) {
-    h->a32.fin = h->f[c];
-    h->a32.fout = h->f[1 - c];
-    return (h->elem == 4 ? launch_step_f32 : launch_step_f16)(
-        h->a32, h->tmap[c], h->p.ctu_order, lim, h->vec, h->grid, h->smem, h->stream);
-  }
-  h->a64.fin = static_cast<const double*>(h->f[c]);
-  h->a64.fout = static_cast<double*>(h->f[1 - c]);
-  return launch_step_f64(h->a64, h->tmap[c], h->p.ctu_order, lim, h->vec, h->grid, h->smem,
-                         h->stream);
+  if (h->elem == 8)
+    return launch_step_f64(h->a64, h->f[c], h->f[1 - c], h->tmap[c], h->p.ctu_order, lim, h->grid,
+                           h->stream);
+  h->a32.fin = h->f[c];
+  h->a32.fout = h->f[1 - c];
+  return (h->elem == 4 ? launch_step_f32 : launch_step_f16)(
+      h->a32, h->tmap[c], h->p.ctu_order, lim, h->vec, h->grid, h->smem, h->stream);
+}
+// The state after n steps.
+void advance(lbm_handle* h, int64_t n) {
+  if (h->elem != 8) h->cur = (int)((h->cur + n) & 1);
+  h->steps += n;
+}
+
+bool add_kernel(cudaGraph_t g, cudaGraphNode_t* prev, void* fn, unsigned grid, unsigned threads,
+                size_t smem, void** args) {
+  cudaKernelNodeParams kp{};
+  kp.func = fn;
+  kp.gridDim = dim3(grid);
+  kp.blockDim = dim3(threads);
+  kp.sharedMemBytes = (unsigned)smem;
+  kp.kernelParams = args;  // copied into the node
+  cudaGraphNode_t node = nullptr;
+  const bool ok = cudaGraphAddKernelNode(&node, g, *prev ? prev : nullptr, *prev ? 1 : 0, &kp) ==
+                  cudaSuccess;
+  *prev = node;
+  return ok;
 }
 
 // A graph of GRAPH_STEPS step kernels chained in order, starting from f[c]:
@@ -632,35 +644,31 @@ cudaError_t launch_one(lbm_handle* h, int c, int lim) {
 // bound by launch overhead).  Built with explicit kernel nodes, so it works
 // on any stream, the legacy default stream included.  nullptr on failure.
 cudaGraphExec_t build_graph(lbm_handle* h, int c, int lim) {
-  const bool f32 = h->elem != 8;
-  const bool regu = h->p.regularize != 0;
-  void* fn = h->elem == 8   ? step_kernel_ptr_f64(h->p.ctu_order, lim, h->vec, regu)
-             : h->elem == 4 ? step_kernel_ptr_f32(h->p.ctu_order, lim, h->vec, regu)
-                            : step_kernel_ptr_f16(h->p.ctu_order, lim, h->vec, regu);
   cudaGraph_t g = nullptr;
   if (cudaGraphCreate(&g, 0) != cudaSuccess) return nullptr;
   cudaGraphNode_t prev = nullptr;
   bool ok = true;
   for (int s = 0; s < GRAPH_STEPS && ok; ++s) {
-    const int cc = (c + s) & 1;
-    StepArgs<float> a32 = h->a32;
-    StepArgs<double> a64 = h->a64;
-    a32.fin = h->f[cc];
-    a32.fout = h->f[1 - cc];
-    a64.fin = static_cast<const double*>(h->f[cc]);
-    a64.fout = static_cast<double*>(h->f[1 - cc]);
-    RowMaps maps = h->tmap[cc];
-    void* args[2] = {f32 ? static_cast<void*>(&a32) : static_cast<void*>(&a64), &maps};
-    cudaKernelNodeParams kp{};
-    kp.func = fn;
-    kp.gridDim = dim3(h->grid);
-    kp.blockDim = dim3(NT);
-    kp.sharedMemBytes = (unsigned)h->smem;
-    kp.kernelParams = args;  // copied into the node
-    cudaGraphNode_t node = nullptr;
-    ok = cudaGraphAddKernelNode(&node, g, prev ? &prev : nullptr, prev ? 1 : 0, &kp) ==
-         cudaSuccess;
-    prev = node;
+    if (h->elem == 8) {
+      const Step64 k = step64(h->a64, h->p.ctu_order, lim);
+      StepArgs<double> in = h->a64, out = h->a64;
+      in.fin = out.fout = h->f[c];
+      in.fout = h->f[1 - c];
+      out.fin = h->f[1 - c];
+      void *a1[] = {&in, &h->tmap[c]}, *a2[] = {&out};
+      ok = add_kernel(g, &prev, k.advect, h->grid, NT, 0, a1) &&
+           add_kernel(g, &prev, k.collide, k.collide_grid, k.collide_threads, 0, a2);
+    } else {
+      const int cc = (c + s) & 1;
+      StepArgs<float> a = h->a32;
+      a.fin = h->f[cc];
+      a.fout = h->f[1 - cc];
+      void* args[] = {&a, &h->tmap[cc]};
+      const bool regu = h->p.regularize != 0;
+      void* fn = (h->elem == 4 ? step_kernel_ptr_f32 : step_kernel_ptr_f16)(h->p.ctu_order, lim,
+                                                                            h->vec, regu);
+      ok = add_kernel(g, &prev, fn, h->grid, NT, h->smem, args);
+    }
   }
   cudaGraphExec_t ex = nullptr;
   if (ok && cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) ex = nullptr;
@@ -689,38 +697,35 @@ int lbm_step(lbm_handle* h, int64_t n) {
       for (; n >= GRAPH_STEPS; n -= GRAPH_STEPS) {
         const cudaError_t e = cudaGraphLaunch(g, h->stream);
         if (e != cudaSuccess) return cuda_check(h, e);
-        h->steps += GRAPH_STEPS;  // an even count: h->cur is unchanged
+        advance(h, GRAPH_STEPS);  // an even count: h->cur is unchanged
       }
     }
   }
   for (int64_t s = 0; s < n; ++s) {
     const cudaError_t e = launch_one(h, h->cur, lim);
     if (e != cudaSuccess) return cuda_check(h, e);
-    h->cur ^= 1;
-    h->steps += 1;
+    advance(h, 1);
   }
   return LBM_OK;
 }
 
+static void apply_geometry(lbm_handle* h, int row_block, int nsm, int ctas) {
+  h->row_block = row_block;
+  h->a64.sub = pick_sub_f64(h->p.Ly, h->nstrip, row_block, nsm);
+  h->grid = grid_for(h, row_block, nsm, ctas);
+  h->a32.row_block = h->a64.row_block = row_block;
+  h->a32.items = h->a64.items = (long long)((h->p.Ly + row_block - 1) / row_block) * h->nstrip;
+}
+
 int lbm_set_launch(lbm_handle* h, int32_t row_block, int32_t ctas_per_sm) {
   if (!h || row_block < 1 || ctas_per_sm < 0) return LBM_ERR_INVALID_ARG;
-  const int lim = h->p.ctu_order == 1 ? 0 : h->p.limiter;
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
-  const bool regu = h->p.regularize != 0;
-  const int occ =
-      h->elem == 4   ? step_occupancy_f32(h->p.ctu_order, lim, h->vec, regu, h->smem)
-      : h->elem == 2 ? step_occupancy_f16(h->p.ctu_order, lim, h->vec, regu, h->smem)
-                     : step_occupancy_f64(h->p.ctu_order, lim, h->vec, regu, h->smem);
+  const int occ = occupancy(h);
   if (nsm < 1 || occ < 1) return set_err(h, LBM_ERR_CUDA);
   if (ctas_per_sm > occ) return LBM_ERR_INVALID_ARG;
   if (ctas_per_sm == 0) ctas_per_sm = occ;
-  const long long items = (long long)((h->p.Ly + row_block - 1) / row_block) * h->nstrip;
-  const long long gmax = (long long)nsm * ctas_per_sm;
-  h->row_block = row_block;
-  h->grid = (int)(items < gmax ? items : gmax);
-  h->a32.row_block = h->a64.row_block = row_block;
-  h->a32.items = h->a64.items = items;
+  apply_geometry(h, row_block, nsm, ctas_per_sm);
   drop_graphs(h);  // built for the old geometry
   return LBM_OK;
 }
@@ -730,25 +735,14 @@ int lbm_tune(lbm_handle* h, int32_t steps_per_trial, lbm_kernel_info* out) {
   const int lim = h->p.ctu_order == 1 ? 0 : h->p.limiter;
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
-  const bool regu = h->p.regularize != 0;
-  const int occ =
-      h->elem == 4   ? step_occupancy_f32(h->p.ctu_order, lim, h->vec, regu, h->smem)
-      : h->elem == 2 ? step_occupancy_f16(h->p.ctu_order, lim, h->vec, regu, h->smem)
-                     : step_occupancy_f64(h->p.ctu_order, lim, h->vec, regu, h->smem);
+  const int occ = occupancy(h);
   if (nsm < 1 || occ < 1) return set_err(h, LBM_ERR_CUDA);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
     return set_err(h, LBM_ERR_CUDA);
   }
-  auto apply = [&](int rb, int ctas) {
-    const long long items = (long long)((h->p.Ly + rb - 1) / rb) * h->nstrip;
-    const long long gmax = (long long)nsm * ctas;
-    h->row_block = rb;
-    h->grid = (int)(items < gmax ? items : gmax);
-    h->a32.row_block = h->a64.row_block = rb;
-    h->a32.items = h->a64.items = items;
-  };
+  auto apply = [&](int rb, int ctas) { apply_geometry(h, rb, nsm, ctas); };
   // one trial: n real steps with geometry (rb, ctas), GPU time in ms
   int r = LBM_OK;
   auto trial = [&](int rb, int ctas, int n, float* ms) -> bool {
@@ -760,8 +754,7 @@ int lbm_tune(lbm_handle* h, int32_t steps_per_trial, lbm_kernel_info* out) {
         r = cuda_check(h, e);
         return false;
       }
-      h->cur ^= 1;
-      h->steps += 1;
+      advance(h, 1);
     }
     cudaEventRecord(e1, h->stream);
     if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(ms, e0, e1) != cudaSuccess) {
@@ -840,7 +833,6 @@ int lbm_step_many(lbm_handle* const* handles, int32_t count, int64_t n) {
     BatchArgs<float>& b = *bp;  // ~23 KB, copied into the launch's parameter space
     long long total = 0;
     b.count = ng;
-    b.sched = h0->d_sched;
     // lattices share the launch, so each keeps row blocks of at least 96 rows
     // (its own may be shorter: sized to fill the GPU alone)
     int rbs[MAXB];
@@ -962,17 +954,14 @@ int lbm_step_diag(lbm_handle* h, int64_t n, double threshold, lbm_diag* out) {
                                                            h->vec, h->grid, h->smem, h->stream);
   } else {
     StepArgs<double> a = h->a64;
-    a.fin = static_cast<const double*>(h->f[h->cur]);
-    a.fout = static_cast<double*>(h->f[1 - h->cur]);
     a.diag_mass = &h->d_acc->mass;
     a.diag_sums = &h->d_acc->nb;
     a.diag_thr = threshold;
-    e = launch_step_f64(a, h->tmap[h->cur], h->p.ctu_order, lim, h->vec, h->grid, h->smem,
-                        h->stream);
+    e = launch_step_f64(a, h->f[h->cur], h->f[1 - h->cur], h->tmap[h->cur], h->p.ctu_order, lim,
+                        h->grid, h->stream);
   }
   if (e != cudaSuccess) return cuda_check(h, e);
-  h->cur ^= 1;
-  h->steps += 1;
+  advance(h, 1);
   if (cuda_check(h, cudaMemcpyAsync(&acc, h->d_acc, sizeof(acc), cudaMemcpyDeviceToHost,
                                     h->stream)) ||
       cuda_check(h, cudaStreamSynchronize(h->stream)))

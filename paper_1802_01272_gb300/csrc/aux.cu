@@ -284,17 +284,8 @@ cudaError_t launch_hist(const AuxArgs& a, const void* f, int nbins, double lo, d
   });
 }
 
-size_t step_smem_bytes(size_t stage_elem, size_t elem) {
-  if (elem == 4)
-    return stage_elem == 2 ? StreamSmem<__half>::bytes() : StreamSmem<float>::bytes();
-  const size_t elems = (size_t)FROWS * FRS + 4 * (size_t)MROWS * MP;  // f*, drho, ux, uy, phi
-  // + 128 bytes to align the staging ring (which also holds the output tiles)
-  // for tensor copies; the fused diagnostics' bubble-site sums, the staging
-  // slots' mbarriers and the CTA's wait-abort flag
-  const size_t scol = stage_elem == 2 ? scol_of<__half>() : scol_of<float>();
-  return 128 + stage_elem * (size_t)NSLOT * RPI * 16 * scol +
-         elem * elems + 6 * sizeof(unsigned long long) + NSLOT * sizeof(unsigned long long) +
-         2 * sizeof(int);
+size_t step_smem_bytes(size_t stage_elem) {
+  return stage_elem == 2 ? StreamSmem<__half>::bytes() : StreamSmem<float>::bytes();
 }
 
 }  // namespace ctulbm

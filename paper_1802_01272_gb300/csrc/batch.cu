@@ -211,7 +211,7 @@ int lbm_batch_create(size_t max_bytes, int32_t chunk_steps, void* cuda_stream, l
     return LBM_ERR_CUDA;
   // the batched kernel's resident CTAs per SM (CTU2 + MC, FP32 storage), two
   // work items of 96 rows x 56 columns each
-  int occ = ctulbm::step_batch_occupancy_f32(2, 0, false, ctulbm::step_smem_bytes(4, 4));
+  int occ = ctulbm::step_batch_occupancy_f32(2, 0, false, ctulbm::step_smem_bytes(4));
   if (occ < 1) occ = 2;
   b->fill_nodes = (long long)nsm * occ * 2 * 96 * 56;
   b->stream = static_cast<cudaStream_t>(cuda_stream);

@@ -26,8 +26,18 @@ struct AuxArgs {
 // lattice has tensor maps (`maps`, for a.fin and a.fout) and stages by them.
 cudaError_t launch_step_f32(const StepArgs<float>& a, const RowMaps& maps, int order, int lim,
                             bool vec, int grid, size_t smem, cudaStream_t s);
-cudaError_t launch_step_f64(const StepArgs<double>& a, const RowMaps& maps, int order, int lim,
-                            bool vec, int grid, size_t smem, cudaStream_t s);
+// The FP64 step: advection from `f` into `work`, collision back into `f`; a.fin
+// and a.fout are ignored.  `maps`: those of f.
+cudaError_t launch_step_f64(const StepArgs<double>& a, void* f, void* work, const RowMaps& maps,
+                            int order, int lim, int grid, cudaStream_t s);
+// Its two kernels, for CUDA graph nodes: advect(StepArgs, RowMaps) on the advection's
+// grid of NT threads, then collide(StepArgs).
+struct Step64 {
+  void *advect, *collide;
+  unsigned collide_grid, collide_threads;
+};
+Step64 step64(const StepArgs<double>& a, int order, int lim);
+int step64_cols();  // columns of a staged box of the advection
 // FP16 shifted storage, FP32 arithmetic (a.fin / a.fout hold half).
 cudaError_t launch_step_f16(const StepArgs<float>& a, const RowMaps& maps, int order, int lim,
                             bool vec, int grid, size_t smem, cudaStream_t s);
@@ -41,17 +51,15 @@ int step_batch_occupancy_f32(int order, int lim, bool regu, size_t smem);
 void* step_batch_kernel_ptr_f32(int order, int lim, bool regu);
 // Largest resident CTAs per SM for the selected step kernel (0 on error).
 int step_occupancy_f32(int order, int lim, bool vec, bool regu, size_t smem);
-int step_occupancy_f64(int order, int lim, bool vec, bool regu, size_t smem);
+int step_occupancy_f64(int order, int lim);  // of the advection kernel
 int step_occupancy_f16(int order, int lim, bool vec, bool regu, size_t smem);
 // The step kernel a launch_step_* call would run (for CUDA graph kernel nodes,
 // whose parameters are (StepArgs, RowMaps) as in a direct launch).
 void* step_kernel_ptr_f32(int order, int lim, bool vec, bool regu);
-void* step_kernel_ptr_f64(int order, int lim, bool vec, bool regu);
 void* step_kernel_ptr_f16(int order, int lim, bool vec, bool regu);
 
-// Dynamic shared memory of the step kernel: staging ring in the storage type
-// (stage_elem bytes per value), the other rings in the arithmetic type.
-size_t step_smem_bytes(size_t stage_elem, size_t elem);
+// Dynamic shared memory of the stream kernel, by storage width (2 or 4 bytes).
+size_t step_smem_bytes(size_t stage_elem);
 
 // f = f^eq(rho, u) - w rho_ref from FP64 device fields.
 cudaError_t launch_init_feq(const AuxArgs& a, void* f, const double* rho, const double* ux,

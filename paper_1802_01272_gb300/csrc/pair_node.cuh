@@ -1,30 +1,44 @@
 // pair_node.cuh -- the per-node part of the step (moments, force, collision)
-// for two x-neighbouring nodes at a time (included by lbm_kernels.cuh inside
-// namespace ctulbm).
+// for one or two x-neighbouring nodes at a time (included by lbm_kernels.cuh
+// inside namespace ctulbm).
 //
-// A value of both nodes is one V = PairOf<T>::type (float2 or double2).  In
-// FP32 every operation on whole pairs is one packed FP32x2 instruction
-// (sm_100+) and every shared-memory access of a pair one 8-byte access, so a
-// pair costs little more issue slots than a node does.
+// N says how many: Pair32 or One64.  A value of the nodes is one N::V (float2 or
+// double).  In FP32 every operation on whole pairs is one
+// packed FP32x2 instruction (sm_100+) and every shared-memory access of a pair one
+// 8-byte access, so a pair costs little more issue slots than a node does.
+struct Pair32 {
+  using T = float;
+  using V = float2;
+  static constexpr int W = 2;
+  static __device__ __forceinline__ V dup(T v) { return make_float2(v, v); }
+  static __device__ __forceinline__ V make(T a, T b) { return make_float2(a, b); }
+  static __device__ __forceinline__ V recip(V v) { return make_float2(rcp(v.x), rcp(v.y)); }
+};
+struct One64 {
+  using T = double;
+  using V = double;
+  static constexpr int W = 1;
+  static __device__ __forceinline__ V dup(T v) { return v; }
+  static __device__ __forceinline__ V recip(V v) { return rcp(v); }
+};
 
-// The constants of the collision phase as pairs.
-template <typename T>
+// The constants of the collision phase.
+template <typename N>
 struct NodeConst {
-  using V = typename PairOf<T>::type;
+  using T = typename N::T;
+  using V = typename N::V;
   V gw1, gw2, gw3, gw4, kw[6];
   V om, ps, p00, p10, pg, p20, p30;
   V lo, hi, nlo, nhi, lo2, hi2;
   V w[3];
-  __device__ explicit NodeConst(const StepArgs<T>& P)
-      : gw1(dup2(P.gw1)), gw2(dup2(P.gw2)), gw3(dup2(P.gw3)), gw4(dup2(P.gw4)), om(dup2(P.omega)),
-        ps(dup2(P.ps)), p00(dup2(P.p00)), p10(dup2(P.p10)), pg(dup2(P.pg)), p20(dup2(P.p20)),
-        p30(dup2(P.p30)), lo(dup2(P.xlo)), hi(dup2(P.xhi)), nlo(dup2(-P.xlo)), nhi(dup2(-P.xhi)),
-        lo2(dup2(P.lo2)), hi2(dup2(P.hi2)) {
+  __device__ explicit NodeConst(const StepArgs<typename N::T>& P)
+      : gw1(N::dup(P.gw1)), gw2(N::dup(P.gw2)), gw3(N::dup(P.gw3)), gw4(N::dup(P.gw4)), om(N::dup(P.omega)),
+        ps(N::dup(P.ps)), p00(N::dup(P.p00)), p10(N::dup(P.p10)), pg(N::dup(P.pg)), p20(N::dup(P.p20)),
+        p30(N::dup(P.p30)), lo(N::dup(P.xlo)), hi(N::dup(P.xhi)), nlo(N::dup(-P.xlo)), nhi(N::dup(-P.xhi)),
+        lo2(N::dup(P.lo2)), hi2(N::dup(P.hi2)) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) kw[i] = dup2(P.kw[i]);
-    w[0] = dup2(P.cls[0].w);
-    w[1] = dup2(P.cls[1].w);  // groups 1 and 2 share their weight
-    w[2] = dup2(P.cls[3].w);
+    for (int i = 0; i < 6; ++i) kw[i] = N::dup(P.kw[i]);
+    for (int i = 0; i < 3; ++i) w[i] = N::dup(P.w[i]);
   }
 };
 
@@ -33,9 +47,8 @@ template <typename V>
 struct Row6 {
   V l, m, r;
 };
-template <typename T>
-__device__ __forceinline__ Row6<typename PairOf<T>::type> row6(const T* p) {
-  using V = typename PairOf<T>::type;
+template <typename V, typename T>
+__device__ __forceinline__ Row6<V> row6(const T* p) {
   return {*reinterpret_cast<const V*>(p - 2), *reinterpret_cast<const V*>(p),
           *reinterpret_cast<const V*>(p + 2)};
 }
@@ -57,35 +70,35 @@ __device__ __forceinline__ Row6<V> sub_rows(const Row6<V>& a, const Row6<V>& b) 
 //    constant vanishes).
 // Both stencils are even across the derivative's direction, so rows are added
 // (for d/dx) or subtracted (for d/dy) first and the sums shared by the pair.
-template <typename T>
-__device__ __forceinline__ void pair_force(const NodeConst<T>& C, const T* const (&ph)[5],
-                                           const T* const (&dq)[5], typename PairOf<T>::type ir,
-                                           typename PairOf<T>::type& gx,
-                                           typename PairOf<T>::type& gy,
-                                           typename PairOf<T>::type& drho) {
-  using V = typename PairOf<T>::type;
-  using PO = PairOf<T>;
-  V px, py;
+template <typename N>
+__device__ __forceinline__ void pair_force(const NodeConst<N>& C, const typename N::T* const (&ph)[5],
+                                           const typename N::T* const (&dq)[5], typename N::V ir,
+                                           typename N::V& gx,
+                                           typename N::V& gy,
+                                           typename N::V& drho) {
+  using T = typename N::T;
+  using V = typename N::V;
+  V px, py, lx, ly;
+  if constexpr (N::W == 2) {
   {
-    const Row6<V> t0 = row6(ph[2]), up = row6(ph[3]), dn = row6(ph[1]);
+    const Row6<V> t0 = row6<V>(ph[2]), up = row6<V>(ph[3]), dn = row6<V>(ph[1]);
     const Row6<V> t1 = add_rows(up, dn), d1 = sub_rows(up, dn);
-    const Row6<V> up2 = row6(ph[4]), dn2 = row6(ph[0]);
+    const Row6<V> up2 = row6<V>(ph[4]), dn2 = row6<V>(ph[0]);
     const Row6<V> d2 = sub_rows(up2, dn2);
     const V t2l = add2(up2.l, dn2.l), t2r = add2(up2.r, dn2.r);
     const V w1 = C.gw1, w2 = C.gw2, w3 = C.gw3, w4 = C.gw4;
     const V al = fma2(w1, t0.l, mul2(w2, t1.l)), am = fma2(w1, t0.m, mul2(w2, t1.m)),
             ar = fma2(w1, t0.r, mul2(w2, t1.r));
     const V bl = fma2(w3, t0.l, mul2(w4, t2l)), br = fma2(w3, t0.r, mul2(w4, t2r));
-    px = sub2(PO::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
-    const V e1 = PO::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d2.r, d2.l);
+    px = sub2(N::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
+    const V e1 = N::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d2.r, d2.l);
     py = sub2(fma2(w1, d1.m, mul2(w2, e1)), fma2(w3, d2.m, mul2(w4, e2)));
   }
-  V lx, ly;
   {
-    const Row6<V> t0 = row6(dq[2]), up = row6(dq[3]), dn = row6(dq[1]);
+    const Row6<V> t0 = row6<V>(dq[2]), up = row6<V>(dq[3]), dn = row6<V>(dq[1]);
     drho = t0.m;
     const Row6<V> t1 = add_rows(up, dn), d1 = sub_rows(up, dn);
-    const Row6<V> up2 = row6(dq[4]), dn2 = row6(dq[0]);
+    const Row6<V> up2 = row6<V>(dq[4]), dn2 = row6<V>(dq[0]);
     const Row6<V> t2 = add_rows(up2, dn2), d2 = sub_rows(up2, dn2);
     const V k0 = C.kw[0], k1 = C.kw[1], k2 = C.kw[2], k3 = C.kw[3], k4 = C.kw[4], k5 = C.kw[5];
     const V al = fma2(k0, t0.l, fma2(k1, t1.l, mul2(k2, t2.l)));
@@ -93,10 +106,35 @@ __device__ __forceinline__ void pair_force(const NodeConst<T>& C, const T* const
     const V ar = fma2(k0, t0.r, fma2(k1, t1.r, mul2(k2, t2.r)));
     const V bl = fma2(k3, t0.l, fma2(k4, t1.l, mul2(k5, t2.l)));
     const V br = fma2(k3, t0.r, fma2(k4, t1.r, mul2(k5, t2.r)));
-    lx = add2(PO::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
-    const V e1 = PO::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d1.r, d1.l);
-    const V h1 = PO::make(d2.m.y + d2.l.y, d2.r.x + d2.m.x), h2 = add2(d2.r, d2.l);
+    lx = add2(N::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
+    const V e1 = N::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d1.r, d1.l);
+    const V h1 = N::make(d2.m.y + d2.l.y, d2.r.x + d2.m.x), h2 = add2(d2.r, d2.l);
     ly = fma2(k0, d1.m, fma2(k1, e1, fma2(k2, e2, fma2(k3, d2.m, fma2(k4, h1, mul2(k5, h2))))));
+  }
+  } else {
+    // one node: columns c - 2 .. c + 2 of five rows
+    const auto diff = [](T a, T b) { return a - b; };
+    {
+      const T* const(&p)[5] = ph;
+      const T x1 = diff(p[2][1], p[2][-1]), x2 = diff(p[2][2], p[2][-2]);
+      const T xd1 = diff(p[3][1] + p[1][1], p[3][-1] + p[1][-1]);
+      const T xd2 = diff(p[4][2] + p[0][2], p[4][-2] + p[0][-2]);
+      px = fma(C.gw1, x1, C.gw2 * xd1) - fma(C.gw3, x2, C.gw4 * xd2);
+      const T y1 = diff(p[3][0], p[1][0]), y2 = diff(p[4][0], p[0][0]);
+      const T yd1 = diff(p[3][1], p[1][1]) + diff(p[3][-1], p[1][-1]);
+      const T yd2 = diff(p[4][2], p[0][2]) + diff(p[4][-2], p[0][-2]);
+      py = fma(C.gw1, y1, C.gw2 * yd1) - fma(C.gw3, y2, C.gw4 * yd2);
+    }
+    {
+      const T* const(&p)[5] = dq;
+      drho = p[2][0];
+      const auto dx = [&](int a, int b) { return (p[2 + b][a] + p[2 - b][a]) - (p[2 + b][-a] + p[2 - b][-a]); };
+      const auto dy = [&](int a, int b) { return (p[2 + b][a] - p[2 - b][a]) + (p[2 + b][-a] - p[2 - b][-a]); };
+      lx = fma(C.kw[0], diff(p[2][1], p[2][-1]), fma(C.kw[1], dx(1, 1), C.kw[2] * dx(1, 2))) +
+           fma(C.kw[3], diff(p[2][2], p[2][-2]), fma(C.kw[4], dx(2, 1), C.kw[5] * dx(2, 2)));
+      ly = fma(C.kw[0], diff(p[3][0], p[1][0]), fma(C.kw[1], dy(1, 1), C.kw[2] * dy(2, 1))) +
+           fma(C.kw[3], diff(p[4][0], p[0][0]), fma(C.kw[4], dy(1, 2), C.kw[5] * dy(2, 2)));
+    }
   }
   gx = fma2(ir, px, lx);
   gy = fma2(ir, py, ly);
@@ -125,24 +163,44 @@ __device__ __forceinline__ GroupSums<V> group_sums(Load f) {
 
 // rho* - rho_ref, u* and p^i - p^w = rho T - [rho T/(1 - b rho) - a rho^2]
 // (Eqs. eder, evdw) of two nodes; f(k) loads velocity k of the pair.
-template <typename T, typename Load>
-__device__ __forceinline__ void pair_moments(const StepArgs<T>& P, Load f,
-                                             typename PairOf<T>::type& dr,
-                                             typename PairOf<T>::type& ux,
-                                             typename PairOf<T>::type& uy,
-                                             typename PairOf<T>::type& phi) {
-  using V = typename PairOf<T>::type;
+template <typename N, typename Load>
+__device__ __forceinline__ void pair_moments(const StepArgs<typename N::T>& P, Load f,
+                                             typename N::V& dr,
+                                             typename N::V& ux,
+                                             typename N::V& uy,
+                                             typename N::V& phi) {
+  using T = typename N::T;
+  using V = typename N::V;
   const GroupSums<V> g = group_sums<V, false>(f);
   dr = add2(g.d[0], add2(g.d[1], add2(g.d[2], g.d[3])));  // the heaviest group last
-  const V rho = add2(dup2(P.rho_ref), dr);
-  const V ir = PairOf<T>::make(rcp(rho.x), rcp(rho.y));
-  const V lo = dup2(P.xlo), hi = dup2(P.xhi);
+  const V rho = add2(N::dup(P.rho_ref), dr);
+  const V ir = N::recip(rho);
+  const V lo = N::dup(P.xlo), hi = N::dup(P.xhi);
   ux = mul2(fma2(lo, add2(g.sx[0], g.sx[2]), mul2(hi, add2(g.sx[1], g.sx[3]))), ir);
   uy = mul2(fma2(lo, add2(g.sy[0], g.sy[1]), mul2(hi, add2(g.sy[2], g.sy[3]))), ir);
-  const V rT = mul2(rho, dup2(P.Tt));
-  const V den = fma2(dup2(P.b), rho, dup2(T(-1)));  // -(1 - b rho)
-  const V q = PairOf<T>::make(rcp(den.x), rcp(den.y));
-  phi = fma2(mul2(dup2(P.a), rho), rho, fma2(rT, q, rT));
+  const V rT = mul2(rho, N::dup(P.Tt));
+  const V den = fma2(N::dup(P.b), rho, N::dup(T(-1)));  // -(1 - b rho)
+  const V q = N::recip(den);
+  phi = fma2(mul2(N::dup(P.a), rho), rho, fma2(rT, q, rT));
+}
+
+// u* alone (rho* known).
+template <typename N, typename Load>
+__device__ __forceinline__ void pair_velocity(const NodeConst<N>& C, Load f,
+                                              typename N::V ir,
+                                              typename N::V& ux,
+                                              typename N::V& uy) {
+  using T = typename N::T;
+  using V = typename N::V;
+  V sx[4], sy[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const V a = sub2(f(4 * m), f(4 * m + 2)), b = sub2(f(4 * m + 1), f(4 * m + 3));
+    sx[m] = sub2(a, b);
+    sy[m] = add2(a, b);
+  }
+  ux = mul2(fma2(C.lo, add2(sx[0], sx[2]), mul2(C.hi, add2(sx[1], sx[3]))), ir);
+  uy = mul2(fma2(C.lo, add2(sy[0], sy[1]), mul2(C.hi, add2(sy[2], sy[3]))), ir);
 }
 
 // The collision as a polynomial in the velocity components.  With x = xi_x,
@@ -159,15 +217,16 @@ struct Poly {
   V c00, c10, c01, c20, c11, c02, c30, c21, c12, c03;
 };
 
-template <typename T>
-__device__ __forceinline__ Poly<typename PairOf<T>::type> collision_poly(
-    const NodeConst<T>& C, typename PairOf<T>::type drho, typename PairOf<T>::type ir,
-    typename PairOf<T>::type u, typename PairOf<T>::type v, typename PairOf<T>::type g,
-    typename PairOf<T>::type h) {
-  using V = typename PairOf<T>::type;
+template <typename N>
+__device__ __forceinline__ Poly<typename N::V> collision_poly(
+    const NodeConst<N>& C, typename N::V drho, typename N::V ir,
+    typename N::V u, typename N::V v, typename N::V g,
+    typename N::V h) {
+  using T = typename N::T;
+  using V = typename N::V;
   const V om = C.om, s = C.ps;
   const V a = fma2(om, u, g), b = fma2(om, v, h);  // w u + dt g
-  const V hu = mul2(mul2(dup2(T(0.5)), u), u), hv = mul2(mul2(dup2(T(0.5)), v), v), uv = mul2(u, v);
+  const V hu = mul2(mul2(N::dup(T(0.5)), u), u), hv = mul2(mul2(N::dup(T(0.5)), v), v), uv = mul2(u, v);
   const V k = add2(hu, hv);                 // u^2 / 2
   const V gu = fma2(g, u, mul2(h, v));      // dt g.u
   const V su = add2(s, hu), sv = add2(s, hv);
@@ -187,8 +246,8 @@ __device__ __forceinline__ Poly<typename PairOf<T>::type> collision_poly(
 }
 
 // Calls put(k, value) with the polynomial's value at velocity k, k = 0 .. 15.
-template <typename T, typename V, typename Put>
-__device__ __forceinline__ void poly_each(const NodeConst<T>& C, const Poly<V>& p, Put put) {
+template <typename N, typename V, typename Put>
+__device__ __forceinline__ void poly_each(const NodeConst<N>& C, const Poly<V>& p, Put put) {
 #pragma unroll
   for (int iy = 0; iy < 2; ++iy) {
     const V y = iy ? C.hi : C.lo, ny = iy ? C.nhi : C.nlo, y2 = iy ? C.hi2 : C.lo2;
@@ -214,42 +273,43 @@ __device__ __forceinline__ void poly_each(const NodeConst<T>& C, const Poly<V>& 
 // collision's with the factor 1 - w, and f^{n+1} = w_k * (the sum) needs f*
 // only through its second and third moments.  p comes in as collision_poly's
 // and leaves as the polynomial of f^{n+1} / w_k (s1 = 1 - w, rw = rho, see pair_collide).
-template <typename T, typename Load>
-__device__ __forceinline__ void regularised_poly(const StepArgs<T>& P, Load f,
-                                                 Poly<typename PairOf<T>::type>& p,
-                                                 typename PairOf<T>::type drho,
-                                                 typename PairOf<T>::type rho,
-                                                 typename PairOf<T>::type u,
-                                                 typename PairOf<T>::type v,
-                                                 typename PairOf<T>::type s1,
-                                                 typename PairOf<T>::type rw) {
-  using V = typename PairOf<T>::type;
+template <typename N, typename Load>
+__device__ __forceinline__ void regularised_poly(const StepArgs<typename N::T>& P, Load f,
+                                                 Poly<typename N::V>& p,
+                                                 typename N::V drho,
+                                                 typename N::V rho,
+                                                 typename N::V u,
+                                                 typename N::V v,
+                                                 typename N::V s1,
+                                                 typename N::V rw) {
+  using T = typename N::T;
+  using V = typename N::V;
   const GroupSums<V> q = group_sums<V, true>(f);
   const T lo = P.xlo, hi = P.xhi, l2 = P.lo2, h2 = P.hi2;
-  auto comb = [&](T a, V x, T b, V y) { return fma2(dup2(a), x, mul2(dup2(b), y)); };
+  auto comb = [&](T a, V x, T b, V y) { return fma2(N::dup(a), x, mul2(N::dup(b), y)); };
   const V mxx = comb(l2, add2(q.d[0], q.d[2]), h2, add2(q.d[1], q.d[3]));
   const V myy = comb(l2, add2(q.d[0], q.d[1]), h2, add2(q.d[2], q.d[3]));
-  const V mxy = fma2(dup2(lo * hi), add2(q.t[1], q.t[2]), comb(l2, q.t[0], h2, q.t[3]));
+  const V mxy = fma2(N::dup(lo * hi), add2(q.t[1], q.t[2]), comb(l2, q.t[0], h2, q.t[3]));
   const V mxxx = comb(lo * l2, add2(q.sx[0], q.sx[2]), hi * h2, add2(q.sx[1], q.sx[3]));
   const V myyy = comb(lo * l2, add2(q.sy[0], q.sy[1]), hi * h2, add2(q.sy[2], q.sy[3]));
   const V mxxy = add2(comb(lo * l2, q.sy[0], hi * h2, q.sy[3]), comb(lo * h2, q.sy[1], hi * l2, q.sy[2]));
   const V mxyy = add2(comb(lo * l2, q.sx[0], hi * h2, q.sx[3]), comb(hi * l2, q.sx[1], lo * h2, q.sx[2]));
-  const V Tt = dup2(P.Tt), ref = dup2(P.rho_ref), half = dup2(T(0.5)), sixth = dup2(T(1) / T(6));
+  const V Tt = N::dup(P.Tt), ref = N::dup(P.rho_ref), half = N::dup(T(0.5)), sixth = N::dup(T(1) / T(6));
   const V uu = mul2(u, u), vv = mul2(v, v), uv = mul2(u, v);
   const V Axx = sub2(add2(mxx, ref), mul2(rho, add2(uu, Tt)));
   const V Ayy = sub2(add2(myy, ref), mul2(rho, add2(vv, Tt)));
   const V Axy = sub2(mxy, mul2(rho, uv));
-  const V T3 = dup2(T(3) * P.Tt);
+  const V T3 = N::dup(T(3) * P.Tt);
   const V ru = mul2(rho, u), rv = mul2(rho, v);
   const V Axxx = sub2(mxxx, mul2(ru, add2(uu, T3))), Ayyy = sub2(myyy, mul2(rv, add2(vv, T3)));
   const V Axxy = sub2(mxxy, mul2(rv, add2(uu, Tt))), Axyy = sub2(mxyy, mul2(ru, add2(vv, Tt)));
   // f^eq / w - rho_ref = drho + rho (P - 1), P - 1 in powers of x, y
-  const V s = dup2(P.ps), hu = mul2(half, uu), hv = mul2(half, vv);
+  const V s = N::dup(P.ps), hu = mul2(half, uu), hv = mul2(half, vv);
   const V k = add2(hu, hv), su = add2(hu, s), sv = add2(hv, s);
-  const V q10 = sub2(dup2(T(1) - T(4) * P.ps), k);
-  const V third = dup2(T(1) / T(3));
+  const V q10 = sub2(N::dup(T(1) - T(4) * P.ps), k);
+  const V third = N::dup(T(1) / T(3));
   Poly<V> r;
-  r.c00 = sub2(sub2(drho, mul2(rho, add2(k, dup2(T(2) * P.ps)))), mul2(half, add2(Axx, Ayy)));
+  r.c00 = sub2(sub2(drho, mul2(rho, add2(k, N::dup(T(2) * P.ps)))), mul2(half, add2(Axx, Ayy)));
   r.c10 = sub2(mul2(ru, q10), mul2(half, add2(Axxx, Axyy)));
   r.c01 = sub2(mul2(rv, q10), mul2(half, add2(Ayyy, Axxy)));
   r.c20 = fma2(rho, su, mul2(half, Axx));
@@ -278,23 +338,24 @@ __device__ __forceinline__ void regularised_poly(const StepArgs<T>& P, Load f,
 // the factors s1 = s (1 - w) and rw = s rho and a constant term: cr = rho_ref
 // (s - 1) / rw (rw = rho_ext to rounding), or rho_ref (s - 1) itself for the
 // regularised collision.
-template <typename T, bool REGU, typename Load, typename Put>
-__device__ __forceinline__ void pair_collide(const StepArgs<T>& P, const NodeConst<T>& C, Load f,
+template <typename N, bool REGU, typename Load, typename Put>
+__device__ __forceinline__ void pair_collide(const StepArgs<typename N::T>& P, const NodeConst<N>& C, Load f,
                                              Put put,
-                                             typename PairOf<T>::type drho,
-                                             typename PairOf<T>::type rho,
-                                             typename PairOf<T>::type ir,
-                                             typename PairOf<T>::type u,
-                                             typename PairOf<T>::type v,
-                                             typename PairOf<T>::type g,
-                                             typename PairOf<T>::type h,
-                                             typename PairOf<T>::type s1,
-                                             typename PairOf<T>::type rw,
-                                             typename PairOf<T>::type cr) {
-  using V = typename PairOf<T>::type;
-  Poly<V> p = collision_poly<T>(C, drho, ir, u, v, g, h);
+                                             typename N::V drho,
+                                             typename N::V rho,
+                                             typename N::V ir,
+                                             typename N::V u,
+                                             typename N::V v,
+                                             typename N::V g,
+                                             typename N::V h,
+                                             typename N::V s1,
+                                             typename N::V rw,
+                                             typename N::V cr) {
+  using T = typename N::T;
+  using V = typename N::V;
+  Poly<V> p = collision_poly<N>(C, drho, ir, u, v, g, h);
   if constexpr (REGU) {
-    regularised_poly<T>(P, f, p, drho, rho, u, v, s1, rw);
+    regularised_poly<N>(P, f, p, drho, rho, u, v, s1, rw);
     p.c00 = add2(p.c00, cr);
     poly_each(C, p, [&](int k, V q) {
       const int grp = k >> 2;

@@ -6,7 +6,7 @@ namespace ctulbm {
 
 #include "step_select.cuh"
 
-using Sel16 = StepSelect<float, __half>;
+using Sel16 = StepSelect<__half>;
 
 cudaError_t launch_step_f16(const StepArgs<float>& a, const RowMaps& maps, int order, int lim,
                             bool vec, int grid, size_t smem, cudaStream_t s) {

@@ -6,7 +6,7 @@ namespace ctulbm {
 
 #include "step_select.cuh"
 
-using Sel32 = StepSelect<float, float>;
+using Sel32 = StepSelect<float>;
 
 cudaError_t launch_step_f32(const StepArgs<float>& a, const RowMaps& maps, int order, int lim,
                             bool vec, int grid, size_t smem, cudaStream_t s) {

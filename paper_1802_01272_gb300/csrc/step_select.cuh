@@ -1,6 +1,6 @@
-// step_select.cuh -- launch-time selection of the step kernel instantiation
-// for one storage type (included by step_fp32.cu, step_fp64.cu, step_fp16.cu
-// inside namespace ctulbm): scheme (CTU1, CTU2 with the MC limiter or with a
+// step_select.cuh -- launch-time selection of the stream kernel instantiation
+// for one storage type (included by step_fp32.cu and step_fp16.cu inside
+// namespace ctulbm): scheme (CTU1, CTU2 with the MC limiter or with a
 // fixed limiter), staging (tensor copies or per-thread loads), fused
 // diagnostics and the regularised collision are compile-time choices, so the
 // plain step's loop carries no code for the others.
@@ -12,14 +12,11 @@ inline bool stream_regs_ok(const void* fn) {
   return cudaFuncGetAttributes(&a, fn) == cudaSuccess && a.numRegs == STREAM_REGS;
 }
 
-template <typename T, typename ST>
+template <typename ST>
 struct StepSelect {
   template <int ORDER, int LIM, bool VEC, bool DIAG, bool REGU>
   static void* ptr() {
-    if constexpr (sizeof(T) == 4)
-      return reinterpret_cast<void*>(&stream_kernel<ST, ORDER, LIM, VEC, DIAG, REGU>);
-    else
-      return reinterpret_cast<void*>(&step_kernel<T, ST, ORDER, LIM, VEC, DIAG, REGU>);
+    return reinterpret_cast<void*>(&stream_kernel<ST, ORDER, LIM, VEC, DIAG, REGU>);
   }
   template <bool VEC, bool DIAG, bool REGU>
   static void* by_scheme(int order, int lim) {
@@ -39,11 +36,11 @@ struct StepSelect {
   static void* select(int order, int lim, bool vec, bool diag, bool regu) {
     return vec ? by_mode<true>(order, lim, diag, regu) : by_mode<false>(order, lim, diag, regu);
   }
-  static cudaError_t launch(const StepArgs<T>& a, const RowMaps& maps, int order, int lim, bool vec,
+  static cudaError_t launch(const StepArgs<float>& a, const RowMaps& maps, int order, int lim, bool vec,
                             int grid, size_t smem, cudaStream_t s) {
     // the shared-memory attribute was set by occupancy() when the handle was made
     void* fn = select(order, lim, vec, a.diag_mass != nullptr, a.regularize != 0);
-    void* args[] = {const_cast<StepArgs<T>*>(&a), const_cast<RowMaps*>(&maps)};
+    void* args[] = {const_cast<StepArgs<float>*>(&a), const_cast<RowMaps*>(&maps)};
     return cudaLaunchKernel(fn, dim3(grid), dim3(NT), args, smem, s);
   }
   // Sets the shared-memory attribute of the plain and fused-diagnostics
@@ -52,7 +49,7 @@ struct StepSelect {
     int occ = 1 << 30;
     for (int d = 0; d < 2; ++d) {
       void* fn = select(order, lim, vec, d == 1, regu);
-      if (sizeof(T) == 4 && !stream_regs_ok(fn)) return 0;
+      if (!stream_regs_ok(fn)) return 0;
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess)
         return 0;

@@ -372,11 +372,6 @@ __device__ __forceinline__ Split<ST> split_of(int x0, int Lx) {
   return {x0 < 0 ? -x0 : min(SCOL, Lx - x0)};
 }
 
-// Row of the lattice that row r of the periodic (or walled) lattice stands for.
-__device__ __forceinline__ int wrap_row(int r, int Ly) {
-  r = r < 0 ? r + Ly : (r >= Ly ? r - Ly : r);
-  return (unsigned)r < (unsigned)Ly ? r : wrapi(r, Ly);  // (lattices lower than a batch)
-}
 // The slot's phase: completed by this arrival and, when the lanes have copies in
 // flight, by their landing.
 __device__ __forceinline__ void lanes_arrive(unsigned bar) {
@@ -630,7 +625,7 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
   while (feed.next(seg)) {
     const StepArgs<float>& P = feed.args(seg);
     const int nit = seg.batches(), x4 = seg.strip * TW + 2 * lane;
-    const NodeConst<float> C(P);
+    const NodeConst<Pair32> C(P);
     float dseg = 0.0f;
     int nseg = 0;
 #pragma unroll 1
@@ -643,7 +638,7 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
         row = row >= SFR ? row - SFR : row;
         const float* src = S.fs + row * (16 * REG) + cm;
         float2 dr, ux, uy, phi;
-        pair_moments<float>(
+        pair_moments<Pair32>(
             P, [&](int k) { return *reinterpret_cast<const float2*>(src + k * REG); }, dr, ux, uy,
             phi);
         if (cm >= MC0 && cm < MC0 + MPP) {
@@ -672,7 +667,7 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
             const float2 rho = add2(dup2(P.rho_ref), *reinterpret_cast<const float2*>(dq[2]));
             const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
             float2 gx, gy, drho;
-            pair_force<float>(C, ph, dq, ir, gx, gy, drho);
+            pair_force<Pair32>(C, ph, dq, ir, gx, gy, drho);
             const float2 u = *reinterpret_cast<const float2*>(S.ux + oc);
             const float2 v = *reinterpret_cast<const float2*>(S.uy + oc);
             const bool in0 = c < seg.ye && x4 < P.Lx, in1 = c < seg.ye && x4 + 1 < P.Lx;
@@ -697,14 +692,14 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
             ST* dst = static_cast<ST*>(P.fout) + (long long)c * P.Lx + x4;
             const unsigned pl = (unsigned)P.plane;
             if constexpr (VEC) {  // Lx is even: a pair is inside or outside
-              pair_collide<float, REGU>(
+              pair_collide<Pair32, REGU>(
                   P, C, load,
                   [&](int k, float2 o) {
                     if (in0) store_pair(dst + (unsigned long long)k * pl, o);
                   },
                   drho, rho, ir, u, v, gx, gy, s1, rw, cr);
             } else {
-              pair_collide<float, REGU>(
+              pair_collide<Pair32, REGU>(
                   P, C, load,
                   [&](int k, float2 o) {
                     if (in0) dst[(unsigned long long)k * pl] = to_store<ST, float>(o.x);

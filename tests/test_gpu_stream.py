@@ -1,4 +1,4 @@
-"""The FP32 / FP16 step kernel at the sizes where its staging, rings and hand-overs
+"""The step kernels at the sizes where their staging, rings, hand-overs and tiles
 can go wrong, against the FP64 oracle: the narrowest lattices with tensor copies
 (68, 72) and widths whose last strip holds 4 columns (116) or all of its 56
 (112); heights under a batch, not a multiple of a batch or of half a batch; row
@@ -34,6 +34,10 @@ CASES = [
     (8, 3, 2, 0, 0, 0, 0, 0),
     (113, 2, 2, 0, 1, 0, 0, 0),
     (57, 30, 1, 0, 0, 0, 1, 5),
+    (16, 8, 2, 0, 0, 0, 0, 0),        # one tile of the FP64 collision, and one node more
+    (17, 9, 2, 0, 0, 0, 0, 0),
+    (84, 40, 2, 0, 1, 0, 0, 33),      # a half strip of the FP64 advection without columns
+    (128, 70, 2, 0, 0, 0, 0, 21),
 ]
 
 
@@ -66,7 +70,7 @@ def _weights(P, O, op):
                       np.zeros((op.Ly, op.Lx)))
 
 
-@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c)))
 def test_against_oracle(P, oracle_mod, case, precision):
     """f after three steps.  FP32: a step rounds each stored value about ten times
@@ -74,9 +78,9 @@ def test_against_oracle(P, oracle_mod, case, precision):
     threefold, and the force adds rounding of the same size: 3 steps x 10 x 3 x
     2^-24 = 5.4e-6 of the largest |f|; bar 1e-5.  FP16: one more rounding of every
     stored deviation per step, 2^-11 of the largest deviation each (and of the
-    start's), passed on at most threefold."""
+    start's), passed on at most threefold.  FP64: 3 x 30 x 2^-53 = 1e-14; bar 1e-13."""
     O = oracle_mod
-    prec = P.LBM_FP32_SHIFTED if precision == "fp32" else P.LBM_FP16_SHIFTED
+    prec = {"fp64": P.LBM_FP64, "fp32": P.LBM_FP32_SHIFTED, "fp16": P.LBM_FP16_SHIFTED}[precision]
     lp = _params(P, case, prec)
     rho, ux, uy = _fields(lp.Lx, lp.Ly)
     op = oracle_params(O, lp)
@@ -90,7 +94,7 @@ def test_against_oracle(P, oracle_mod, case, precision):
         fg = L.get_f()
     fo = O.step(op, f0, STEPS)
     err = np.abs(fg - fo).max()
-    bar = 1e-5 * np.abs(fo).max()
+    bar = (1e-13 if precision == "fp64" else 1e-5) * np.abs(fo).max()
     if precision == "fp16":
         # f - w rho_ref with w from f^eq at rest at T = 1 (= w rho)
         op1 = oracle_params(O, lp)
