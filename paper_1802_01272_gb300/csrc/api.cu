@@ -156,8 +156,6 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   a.Ly = p.Ly;
   a.plane = (long long)p.Lx * p.Ly;
   a.nstrip = h->nstrip;
-  a.row_block = h->row_block;
-  a.items = (long long)((p.Ly + h->row_block - 1) / h->row_block) * h->nstrip;
   a.diag_mass = nullptr;
   a.diag_sums = nullptr;
   a.diag_thr = (T)0;
@@ -381,6 +379,27 @@ int grid_for(const lbm_handle* h, long long rb, int nsm, int ctas) {
   return (int)(want < gmax ? want : gmax);
 }
 
+// Row blocks of rb rows on at most ctas CTAs per SM.
+void apply_geometry(lbm_handle* h, int rb, int nsm, int ctas) {
+  h->row_block = rb;
+  h->a64.sub = pick_sub_f64(h->p.Ly, h->nstrip, rb, nsm);
+  h->grid = grid_for(h, rb, nsm, ctas);
+  h->a32.row_block = h->a64.row_block = rb;
+  h->a32.items = h->a64.items = (long long)((h->p.Ly + rb - 1) / rb) * h->nstrip;
+  if (h->elem == 8) return;
+  // A launch that leaves SMs without a CTA is bound by one item's latency: its blocks
+  // are handed out in parts of 8 or 4 rows while there is an SM for each (128 x 8:
+  // 7.3 us per step in one part of 8 rows per strip, 6.0 in two of 4).
+  for (int part = 8; part >= 4; part /= 2) {
+    const long long n = (long long)((h->p.Ly + part - 1) / part) * h->nstrip;
+    if (rb > part && rb % part == 0 && n <= nsm) {
+      h->a32.row_block = part;
+      h->a32.items = n;
+      h->grid = (int)n;
+    }
+  }
+}
+
 int check_device_error(lbm_handle* h) {
   unsigned int e = 0;
   if (cudaMemcpyAsync(&e, h->d_err, sizeof(e), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
@@ -481,12 +500,11 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
   }
   h->row_block = (int)(h->elem == 8 ? pick_row_block_f64(p->Ly, h->nstrip, nsm)
                                     : pick_row_block(p->Ly, h->nstrip, (long long)nsm * occ));
-  h->a64.sub = pick_sub_f64(p->Ly, h->nstrip, h->row_block, nsm);
-  h->grid = grid_for(h, h->row_block, nsm, occ);
   if (h->elem == 8)
     fill_step_args<double>(h, h->a64);
   else
     fill_step_args<float>(h, h->a32);
+  apply_geometry(h, h->row_block, nsm, occ);
   h->a32.tma_in = h->a64.tma_in = tin;
   AuxArgs& x = h->aux;
   x.Lx = p->Lx;
@@ -624,17 +642,22 @@ void advance(lbm_handle* h, int64_t n) {
   h->steps += n;
 }
 
+// Chains a kernel to the graph by a programmatic edge (as launch_dependent).
 bool add_kernel(cudaGraph_t g, cudaGraphNode_t* prev, void* fn, unsigned grid, unsigned threads,
                 size_t smem, void** args) {
-  cudaKernelNodeParams kp{};
-  kp.func = fn;
-  kp.gridDim = dim3(grid);
-  kp.blockDim = dim3(threads);
-  kp.sharedMemBytes = (unsigned)smem;
-  kp.kernelParams = args;  // copied into the node
+  cudaGraphNodeParams np{};
+  np.type = cudaGraphNodeTypeKernel;
+  np.kernel.func = fn;
+  np.kernel.gridDim = dim3(grid);
+  np.kernel.blockDim = dim3(threads);
+  np.kernel.sharedMemBytes = (unsigned)smem;
+  np.kernel.kernelParams = args;  // copied into the node
+  cudaGraphEdgeData edge{};
+  edge.from_port = cudaGraphKernelNodePortProgrammatic;
+  edge.type = cudaGraphDependencyTypeProgrammatic;
   cudaGraphNode_t node = nullptr;
-  const bool ok = cudaGraphAddKernelNode(&node, g, *prev ? prev : nullptr, *prev ? 1 : 0, &kp) ==
-                  cudaSuccess;
+  const bool ok = cudaGraphAddNode(&node, g, *prev ? prev : nullptr, *prev ? &edge : nullptr,
+                                   *prev ? 1 : 0, &np) == cudaSuccess;
   *prev = node;
   return ok;
 }
@@ -707,14 +730,6 @@ int lbm_step(lbm_handle* h, int64_t n) {
     advance(h, 1);
   }
   return LBM_OK;
-}
-
-static void apply_geometry(lbm_handle* h, int row_block, int nsm, int ctas) {
-  h->row_block = row_block;
-  h->a64.sub = pick_sub_f64(h->p.Ly, h->nstrip, row_block, nsm);
-  h->grid = grid_for(h, row_block, nsm, ctas);
-  h->a32.row_block = h->a64.row_block = row_block;
-  h->a32.items = h->a64.items = (long long)((h->p.Ly + row_block - 1) / row_block) * h->nstrip;
 }
 
 int lbm_set_launch(lbm_handle* h, int32_t row_block, int32_t ctas_per_sm) {
@@ -833,14 +848,26 @@ int lbm_step_many(lbm_handle* const* handles, int32_t count, int64_t n) {
     BatchArgs<float>& b = *bp;  // ~23 KB, copied into the launch's parameter space
     long long total = 0;
     b.count = ng;
-    // lattices share the launch, so each keeps row blocks of at least 96 rows
-    // (its own may be shorter: sized to fill the GPU alone)
-    int rbs[MAXB];
-    long long its[MAXB];
+    // row blocks: one height for all, as pick_row_block chooses it for one lattice
+    int rb = 16;
+    long long best = 0, its[MAXB];
+    for (int r = 16; r <= 1024; r += 4) {
+      long long items = 0;
+      int most = 0;
+      for (int i = 0; i < ng; ++i) {
+        const int Ly = group[i]->a32.Ly;
+        items += (long long)((Ly + r - 1) / r) * group[i]->nstrip;
+        most = Ly > most ? Ly : most;
+      }
+      const long long cost = (items + grid_max - 1) / grid_max * (r + 8);
+      if (best == 0 || cost < best) {
+        best = cost;
+        rb = r;
+      }
+      if (r >= most) break;
+    }
     for (int i = 0; i < ng; ++i) {
-      const StepArgs<float>& a = group[i]->a32;
-      rbs[i] = a.row_block < 96 ? (a.Ly < 96 ? a.Ly : 96) : a.row_block;
-      its[i] = (long long)((a.Ly + rbs[i] - 1) / rbs[i]) * a.nstrip;
+      its[i] = (long long)((group[i]->a32.Ly + rb - 1) / rb) * group[i]->nstrip;
       b.item_start[i] = total;
       total += its[i];
     }
@@ -853,7 +880,7 @@ int lbm_step_many(lbm_handle* const* handles, int32_t count, int64_t n) {
         lbm_handle* h = group[i];
         const int c = (h->cur + s) & 1;
         b.L[i] = h->a32;
-        b.L[i].row_block = rbs[i];
+        b.L[i].row_block = rb;
         b.L[i].items = its[i];
         b.L[i].fin = static_cast<const float*>(h->f[c]);
         b.L[i].fout = static_cast<float*>(h->f[1 - c]);
@@ -877,16 +904,7 @@ int lbm_step_many(lbm_handle* const* handles, int32_t count, int64_t n) {
       for (int s = 0; s < GRAPH_STEPS && ok; ++s) {
         args_for(s);
         void* kargs[1] = {&b};
-        cudaKernelNodeParams kp{};
-        kp.func = fn;
-        kp.gridDim = dim3(g);
-        kp.blockDim = dim3(NT);
-        kp.sharedMemBytes = (unsigned)group[0]->smem;
-        kp.kernelParams = kargs;  // copied into the node
-        cudaGraphNode_t node = nullptr;
-        ok = cudaGraphAddKernelNode(&node, gr, prev ? &prev : nullptr, prev ? 1 : 0, &kp) ==
-             cudaSuccess;
-        prev = node;
+        ok = add_kernel(gr, &prev, fn, g, NT, group[0]->smem, kargs);
       }
       if (ok) ok = cudaGraphInstantiate(&ex, gr, 0) == cudaSuccess;
       if (gr) cudaGraphDestroy(gr);

@@ -22,6 +22,23 @@ struct AuxArgs {
   float xif[16][2], wf[16];  // the same tables rounded to float on the host
 };
 
+// Launch with programmatic dependence on the stream's previous launch (see
+// previous_step_done).
+inline cudaError_t launch_dependent(const void* fn, unsigned grid, unsigned threads, size_t smem,
+                                    cudaStream_t s, void** args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelExC(&c, fn, args);
+}
+
 // One fused step kernel: returns cudaSuccess or the launch error.  `vec`: the
 // lattice has tensor maps (`maps`, for a.fin and a.fout) and stages by them.
 cudaError_t launch_step_f32(const StepArgs<float>& a, const RowMaps& maps, int order, int lim,

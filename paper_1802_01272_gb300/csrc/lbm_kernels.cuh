@@ -241,6 +241,28 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
+// Steps are launched with programmatic dependence (launch_dependent): a step's CTAs
+// come up, set up their barriers and fetch parameters and tensor maps while the last
+// of the step before end; they touch nothing that a launch before them writes or
+// reads until those have completed.  (Also correct after any other launch.)  The
+// launch is not let go earlier, by griddepcontrol.launch_dependents: CTAs that wait
+// on an SM displace and unbalance those still to come (256^2 10.3 -> 11.8 us per step,
+// 1024^2 FP64 970 -> 1160); without programmatic dependence 256^2 takes 10.8, 128^2
+// FP64 25.6 against 25.1.
+__device__ __forceinline__ void previous_step_done() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+// A value the compiler does not know: a counter that starts here keeps its loop from
+// being peeled into copies for the first iterations, each of which would have to be
+// fetched once per launch.
+__device__ __forceinline__ int unknown(int v) {
+  int r;
+  asm volatile("mov.b32 %0, %1;\n" : "=r"(r) : "r"(v));
+  return r;
+}
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];\n" ::"l"(map) : "memory");
+}
 // One tensor copy from row y.. of plane k of the (x, plane, row) tensor into `dst`.
 __device__ __forceinline__ void tma_load_tile(void* dst, const CUtensorMap* map, int x, int k, int y,
                                               unsigned long long* bar) {

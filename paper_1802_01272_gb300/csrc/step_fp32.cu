@@ -50,7 +50,7 @@ cudaError_t launch_step_batch_f32(const BatchArgs<float>& b, int order, int lim,
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<BatchArgs<float>*>(&b)};
-  return cudaLaunchKernel(fn, dim3(grid), dim3(NT), args, smem, s);
+  return launch_dependent(fn, grid, NT, smem, s, args);
 }
 
 void* step_batch_kernel_ptr_f32(int order, int lim, bool regu) {

@@ -42,10 +42,10 @@ cudaError_t launch_step_f64(const StepArgs<double>& a, void* f, void* work, cons
   in.fout = work;
   out.fin = work;
   void* args[] = {&in, const_cast<RowMaps*>(&maps)};
-  const cudaError_t e = cudaLaunchKernel(k.advect, dim3(grid), dim3(NT), args, 0, s);
+  const cudaError_t e = launch_dependent(k.advect, grid, NT, 0, s, args);
   if (e != cudaSuccess) return e;
   void* args2[] = {&out};
-  return cudaLaunchKernel(k.collide, dim3(k.collide_grid), dim3(k.collide_threads), args2, 0, s);
+  return launch_dependent(k.collide, k.collide_grid, k.collide_threads, 0, s, args2);
 }
 
 int step_occupancy_f64(int order, int lim) {

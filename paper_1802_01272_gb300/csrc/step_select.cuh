@@ -41,7 +41,7 @@ struct StepSelect {
     // the shared-memory attribute was set by occupancy() when the handle was made
     void* fn = select(order, lim, vec, a.diag_mass != nullptr, a.regularize != 0);
     void* args[] = {const_cast<StepArgs<float>*>(&a), const_cast<RowMaps*>(&maps)};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(NT), args, smem, s);
+    return launch_dependent(fn, grid, NT, smem, s, args);
   }
   // Sets the shared-memory attribute of the plain and fused-diagnostics
   // variants; returns the CTAs per SM both reach (0 on error).

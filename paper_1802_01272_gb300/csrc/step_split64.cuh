@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(NT, 2)
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncwarp();
+  previous_step_done();
   const int Lx = P.Lx, Ly = P.Ly;
   unsigned phase = 0;
   bool dead = false;  // a staged batch did not arrive: the results are void, nothing more is staged
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(C64_NT)
   const int x0 = bx * C64_TX, y0 = by * C64_TY;
   const double* const fin = static_cast<const double*>(P.fin);
   const long long pl = P.plane;
+  previous_step_done();
   for (int e = tid; e < C64_PX * C64_PY; e += C64_NT) {
     const int iy = e / C64_PX, ix = e - iy * C64_PX;
     const int row = y0 - 2 + iy, x = wrapi(x0 - 2 + ix, Lx);

@@ -387,16 +387,21 @@ static __device__ __forceinline__ void stage_chunks(ST* dst, unsigned bar, Split
                                                     const ST* fin, long long plane, int x0, int r0,
                                                     int Lx, int Ly, int walls) {
   constexpr int E = 16 / (int)sizeof(ST), N = StreamLayout<ST>::SCOL / E;
-#pragma unroll 1
-  for (int e = threadIdx.x & 31; e < SR * 4 * N; e += 32) {
-    const int rg = e / N, j = (e - rg * N) * E, row = r0 + (rg >> 2);
-    if (walls && (unsigned)row >= (unsigned)Ly) continue;
-    const int x = x0 + j;
-    const ST* p = fin + 4 * (rg & 3) * plane + (long long)wrap_row(row, Ly) * Lx +
-                  (x < 0 ? x + Lx : (x >= Lx ? x - Lx : x));
+  const int lane = threadIdx.x & 31;
+  const auto copy = [&](int rg, int x, int j, const ST* row) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst + split.at(rg, j))),
-                 "l"(p)
+                 "l"(row + 4 * (rg & 3) * plane + x)
                  : "memory");
+  };
+#pragma unroll
+  for (int r = 0; r < SR; ++r) {
+    if (walls && (unsigned)(r0 + r) >= (unsigned)Ly) continue;
+    const ST* row = fin + (long long)wrap_row(r0 + r, Ly) * Lx;
+#pragma unroll
+    for (int e = lane; e < 4 * N; e += 32) {
+      const int grp = e / N, j = (e - grp * N) * E, x = x0 + j;
+      copy(4 * r + grp, x < 0 ? x + Lx : (x >= Lx ? x - Lx : x), j, row);
+    }
   }
   lanes_arrive(bar);
 }
@@ -538,7 +543,7 @@ __device__ __forceinline__ void advect_role(Feed feed, const StreamSmem<ST>& S, 
   // this lane's velocities: groups h and h + 2 (equal |xi_x|) of the quadrant
   float* const dst0 = S.fs + (4 * h + q) * REG + col;
   constexpr int D2 = 8 * REG;  // f* ring: group h + 2
-  unsigned g = 0;
+  unsigned g = (unsigned)unknown(0);  // batches so far
   int ring = 0;
   Segment seg;
   while (feed.next(seg)) {
@@ -629,117 +634,121 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
     float dseg = 0.0f;
     int nseg = 0;
 #pragma unroll 1
-    for (int it = 0; it < nit; ++it, ++g) {
+    for (int it = unknown(0); it < nit; ++it, ++g) {
       role_wait(BAR_FULL + (g & 1));
       const int c0 = seg.ys + RPI * (it - WARM);  // first output row of this batch
-      if (it >= 1) {
-        // moments of row B - 2 + w
-        int row = ring + w;
-        row = row >= SFR ? row - SFR : row;
-        const float* src = S.fs + row * (16 * REG) + cm;
-        float2 dr, ux, uy, phi;
-        pair_moments<Pair32>(
-            P, [&](int k) { return *reinterpret_cast<const float2*>(src + k * REG); }, dr, ux, uy,
-            phi);
-        if (cm >= MC0 && cm < MC0 + MPP) {
-          const int m = (mring + w) * MPP + cm - MC0, mu = row * MPP + cm - MC0;
-          *reinterpret_cast<float2*>(S.drho + m) = dr;
-          *reinterpret_cast<float2*>(S.phi + m) = phi;
-          *reinterpret_cast<float2*>(S.ux + mu) = ux;
-          *reinterpret_cast<float2*>(S.uy + mu) = uy;
-        }
-        if (it >= WARM) {
-          collide_barrier();
-          const int c = c0 + w;  // this warp's row
-          float2 post = dup2(-1.0f);
-          if (lane < TW / 2) {
-            const float *ph[5], *dq[5];
+      // moments of row B - 2 + w (those of a segment's first batch are void: a branch
+      // around them would give the loop a second copy to fetch)
+      int row = ring + w;
+      row = row >= SFR ? row - SFR : row;
+      const float* src = S.fs + row * (16 * REG) + cm;
+      float2 dr, ux, uy, phi;
+      pair_moments<Pair32>(
+          P, [&](int k) { return *reinterpret_cast<const float2*>(src + k * REG); }, dr, ux, uy,
+          phi);
+      if (cm >= MC0 && cm < MC0 + MPP) {
+        const int m = (mring + w) * MPP + cm - MC0, mu = row * MPP + cm - MC0;
+        *reinterpret_cast<float2*>(S.drho + m) = dr;
+        *reinterpret_cast<float2*>(S.phi + m) = phi;
+        *reinterpret_cast<float2*>(S.ux + mu) = ux;
+        *reinterpret_cast<float2*>(S.uy + mu) = uy;
+      }
+      if (it >= WARM) {
+        collide_barrier();
+        const int c = c0 + w;  // this warp's row
+        float2 post = dup2(-1.0f);
+        if (lane < TW / 2) {
+          const float *ph[5], *dq[5];
 #pragma unroll
-            for (int b = 0; b < 5; ++b) {  // rows c - 2 .. c + 2 = (B - 2 + w) - 4 .. + 0
-              const unsigned o = (unsigned)(mring + w + b + SMR - 4) * MPP;
-              const unsigned r = min(o, o - SMR * MPP) + cc - MC0;  // mod SMR rows
-              ph[b] = S.phi + r;
-              dq[b] = S.drho + r;
-            }
-            int frow = ring + SFR - 2 + w;
-            frow = frow >= SFR ? frow - SFR : frow;
-            const int oc = frow * MPP + cc - MC0;
-            const float2 rho = add2(dup2(P.rho_ref), *reinterpret_cast<const float2*>(dq[2]));
-            const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
-            float2 gx, gy, drho;
-            pair_force<Pair32>(C, ph, dq, ir, gx, gy, drho);
-            const float2 u = *reinterpret_cast<const float2*>(S.ux + oc);
-            const float2 v = *reinterpret_cast<const float2*>(S.uy + oc);
-            const bool in0 = c < seg.ye && x4 < P.Lx, in1 = c < seg.ye && x4 + 1 < P.Lx;
-            if ((in0 && !(rho.x > 0.0f && rho.x < 1e30f)) ||
-                (in1 && !(rho.y > 0.0f && rho.y < 1e30f)))
-              atomicOr(P.err, 1u);
-            float2 s1 = dup2(P.one_m_omega), rw = rho, cr = dup2(0.0f);
-            if (P.reservoir) {
-              // outside R_BC the node is rescaled to rho_ext, s = rho_ext / rho
-              const float dx = (float)x4 - P.cxc, dy = (float)c - P.cyc;
-              const auto rescale = [&](float& a, float& b, float& e, float i) {
-                const float s = P.rho_ext * i;
-                a *= s;
-                b *= s;  // (not rho_ext: s must scale mass and momentum alike)
-                e = P.rho_ref * (s - 1.0f) * (REGU ? 1.0f : P.irho_ext);
-              };
-              if (dx * dx + dy * dy > P.rbc2) rescale(s1.x, rw.x, cr.x, ir.x);
-              if ((dx + 1.0f) * (dx + 1.0f) + dy * dy > P.rbc2) rescale(s1.y, rw.y, cr.y, ir.y);
-            }
-            const float* fsrc = S.fs + frow * (16 * REG) + cc;
-            auto load = [&](int k) { return *reinterpret_cast<const float2*>(fsrc + k * REG); };
-            ST* dst = static_cast<ST*>(P.fout) + (long long)c * P.Lx + x4;
-            const unsigned pl = (unsigned)P.plane;
-            if constexpr (VEC) {  // Lx is even: a pair is inside or outside
-              pair_collide<Pair32, REGU>(
-                  P, C, load,
-                  [&](int k, float2 o) {
-                    if (in0) store_pair(dst + (unsigned long long)k * pl, o);
-                  },
-                  drho, rho, ir, u, v, gx, gy, s1, rw, cr);
-            } else {
-              pair_collide<Pair32, REGU>(
-                  P, C, load,
-                  [&](int k, float2 o) {
-                    if (in0) dst[(unsigned long long)k * pl] = to_store<ST, float>(o.x);
-                    if (in1) dst[(unsigned long long)k * pl + 1] = to_store<ST, float>(o.y);
-                  },
-                  drho, rho, ir, u, v, gx, gy, s1, rw, cr);
-            }
-            if (DIAG) post = make_float2(in0 ? rw.x : -1.0f, in1 ? rw.y : -1.0f);
+          for (int b = 0; b < 5; ++b) {  // rows c - 2 .. c + 2 = (B - 2 + w) - 4 .. + 0
+            const unsigned o = (unsigned)(mring + w + b + SMR - 4) * MPP;
+            const unsigned r = min(o, o - SMR * MPP) + cc - MC0;  // mod SMR rows
+            ph[b] = S.phi + r;
+            dq[b] = S.drho + r;
           }
-          if (DIAG) {  // fused diagnostics: mass per thread, bubble sites per warp
-            unsigned long long a[6] = {0, 0, 0, 0, 0, 0};
-            bool any = false;
+          int frow = ring + SFR - 2 + w;
+          frow = frow >= SFR ? frow - SFR : frow;
+          const int oc = frow * MPP + cc - MC0;
+          const float2 rho = add2(dup2(P.rho_ref), *reinterpret_cast<const float2*>(dq[2]));
+          const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
+          float2 gx, gy, drho;
+          pair_force<Pair32>(C, ph, dq, ir, gx, gy, drho);
+          const float2 u = *reinterpret_cast<const float2*>(S.ux + oc);
+          const float2 v = *reinterpret_cast<const float2*>(S.uy + oc);
+          const bool in0 = c < seg.ye && x4 < P.Lx, in1 = c < seg.ye && x4 + 1 < P.Lx;
+          if ((in0 && !(rho.x > 0.0f && rho.x < 1e30f)) ||
+              (in1 && !(rho.y > 0.0f && rho.y < 1e30f)))
+            atomicOr(P.err, 1u);
+          float2 s1 = dup2(P.one_m_omega), rw = rho, cr = dup2(0.0f);
+          if (P.reservoir) {
+            // outside R_BC the node is rescaled to rho_ext, s = rho_ext / rho
+            const float dx = (float)x4 - P.cxc, dy = (float)c - P.cyc;
+            const auto rescale = [&](float& a, float& b, float& e, float i) {
+              const float s = P.rho_ext * i;
+              a *= s;
+              b *= s;  // (not rho_ext: s must scale mass and momentum alike)
+              e = P.rho_ref * (s - 1.0f) * (REGU ? 1.0f : P.irho_ext);
+            };
+            if (dx * dx + dy * dy > P.rbc2) rescale(s1.x, rw.x, cr.x, ir.x);
+            if ((dx + 1.0f) * (dx + 1.0f) + dy * dy > P.rbc2) rescale(s1.y, rw.y, cr.y, ir.y);
+          }
+          const float* fsrc = S.fs + frow * (16 * REG) + cc;
+          auto load = [&](int k) { return *reinterpret_cast<const float2*>(fsrc + k * REG); };
+          // plane k of the pair: one widening multiply-add per store
+          char* const dst0 = static_cast<char*>(P.fout) +
+                             (unsigned long long)((unsigned)c * (unsigned)P.Lx + (unsigned)x4) * sizeof(ST);
+          const auto at = [&](int k) {
+            return reinterpret_cast<ST*>(
+                dst0 + (unsigned long long)(unsigned)P.plane * (unsigned)(k * sizeof(ST)));
+          };
+          if constexpr (VEC) {  // Lx is even: a pair is inside or outside
+            pair_collide<Pair32, REGU>(
+                P, C, load,
+                [&](int k, float2 o) {
+                  if (in0) store_pair(at(k), o);
+                },
+                drho, rho, ir, u, v, gx, gy, s1, rw, cr);
+          } else {
+            pair_collide<Pair32, REGU>(
+                P, C, load,
+                [&](int k, float2 o) {
+                  if (in0) at(k)[0] = to_store<ST, float>(o.x);
+                  if (in1) at(k)[1] = to_store<ST, float>(o.y);
+                },
+                drho, rho, ir, u, v, gx, gy, s1, rw, cr);
+          }
+          if (DIAG) post = make_float2(in0 ? rw.x : -1.0f, in1 ? rw.y : -1.0f);
+        }
+        if (DIAG) {  // fused diagnostics: mass per thread, bubble sites per warp
+          unsigned long long a[6] = {0, 0, 0, 0, 0, 0};
+          bool any = false;
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float p = e ? post.y : post.x;
-              if (p >= 0.0f) {
-                dseg += p - P.rho_ref;
-                ++nseg;
-                if (p < P.diag_thr) {
-                  const unsigned long long i = (unsigned long long)(x4 + e), j = (unsigned long long)c;
-                  any = true;
-                  a[0] += 1;
-                  a[1] += i;
-                  a[2] += j;
-                  a[3] += i * i;
-                  a[4] += i * j;
-                  a[5] += j * j;
-                }
+          for (int e = 0; e < 2; ++e) {
+            const float p = e ? post.y : post.x;
+            if (p >= 0.0f) {
+              dseg += p - P.rho_ref;
+              ++nseg;
+              if (p < P.diag_thr) {
+                const unsigned long long i = (unsigned long long)(x4 + e), j = (unsigned long long)c;
+                any = true;
+                a[0] += 1;
+                a[1] += i;
+                a[2] += j;
+                a[3] += i * i;
+                a[4] += i * j;
+                a[5] += j * j;
               }
             }
-            if (__ballot_sync(0xffffffffu, any)) {  // bubble sites are rare: sum them only here
+          }
+          if (__ballot_sync(0xffffffffu, any)) {  // bubble sites are rare: sum them only here
 #pragma unroll
-              for (int o = 16; o > 0; o >>= 1) {
+            for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-                for (int t = 0; t < 6; ++t) a[t] += __shfl_down_sync(0xffffffffu, a[t], o);
-              }
-              if (lane == 0) {
+              for (int t = 0; t < 6; ++t) a[t] += __shfl_down_sync(0xffffffffu, a[t], o);
+            }
+            if (lane == 0) {
 #pragma unroll
-                for (int t = 0; t < 6; ++t) atomicAdd(&S.dsums[t], a[t]);
-              }
+              for (int t = 0; t < 6; ++t) atomicAdd(&S.dsums[t], a[t]);
             }
           }
         }
@@ -777,7 +786,9 @@ __global__ void __launch_bounds__(NT, STREAM_CTAS)
     stream_kernel(const __grid_constant__ StepArgs<float> P, const __grid_constant__ RowMaps maps) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const StreamSmem<ST> S(smem_raw);
+  if (VEC && threadIdx.x == 0) prefetch_map(maps.m);
   S.init();
+  previous_step_done();
   double dmass = 0.0;  // fused diagnostics: this thread's mass over all its segments
   stream_roles<ORDER, LIM, ST, VEC, DIAG, REGU>(SingleFeed(P, maps), S, dmass);
   if (DIAG) {
@@ -798,6 +809,7 @@ __global__ void __launch_bounds__(NT, STREAM_CTAS)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const StreamSmem<float> S(smem_raw);
   S.init();
+  previous_step_done();
   double dmass = 0.0;  // unused: batched launches carry no fused diagnostics
   stream_roles<ORDER, LIM, float, true, false, REGU>(BatchFeed(B), S, dmass);
 }
