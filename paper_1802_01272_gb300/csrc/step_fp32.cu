@@ -62,7 +62,7 @@ int step_batch_occupancy_f32(int order, int lim, bool regu, size_t smem) {
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return 0;
-  if (!stream_regs_ok(fn)) return 0;
+  if (!stream_regs_ok(fn, regu)) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, NT, smem) != cudaSuccess) return 0;
   return n;

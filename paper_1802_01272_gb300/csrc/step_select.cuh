@@ -6,10 +6,10 @@
 // plain step's loop carries no code for the others.
 #pragma once
 
-// The stream kernel's roles trade registers, which must add up (see STREAM_REGS).
-inline bool stream_regs_ok(const void* fn) {
+// The stream kernel's roles trade registers, which must add up (see StreamRegs).
+inline bool stream_regs_ok(const void* fn, bool regu) {
   cudaFuncAttributes a;
-  return cudaFuncGetAttributes(&a, fn) == cudaSuccess && a.numRegs == STREAM_REGS;
+  return cudaFuncGetAttributes(&a, fn) == cudaSuccess && a.numRegs == (regu ? StreamRegs<true>::LAUNCH : StreamRegs<false>::LAUNCH);
 }
 
 template <typename ST>
@@ -49,7 +49,7 @@ struct StepSelect {
     int occ = 1 << 30;
     for (int d = 0; d < 2; ++d) {
       void* fn = select(order, lim, vec, d == 1, regu);
-      if (!stream_regs_ok(fn)) return 0;
+      if (!stream_regs_ok(fn, regu)) return 0;
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess)
         return 0;

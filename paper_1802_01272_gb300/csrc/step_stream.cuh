@@ -48,12 +48,17 @@ constexpr int SNS = 2;                 // staging slots per advect warp: the hal
 constexpr int SFR = 10;                // f* ring (and u*): rows B - 4 .. B + 5
 constexpr int SMR = 12;                // rho* and p^i - p^w rings: rows B - 6 .. B + 5
 constexpr int MC0 = 2, MPP = 60;       // region columns 2 .. 61 of the moments are kept
-// Registers per thread at launch (three CTAs of 256 threads fit an SM's 65536)
-// and after the roles have traded them: the advect warps take what the collide
-// warps give up, no more (a larger sum would wait for registers forever; the
-// host refuses a kernel that was not compiled to STREAM_REGS).
-constexpr int STREAM_CTAS = 3, STREAM_REGS = 80, ADVECT_REGS = 96, COLLIDE_REGS = 64;
-static_assert(ADVECT_REGS + COLLIDE_REGS == 2 * STREAM_REGS, "");
+// Resident CTAs per SM, registers per thread at launch, and after the roles have
+// traded them: the advect warps take what the collide warps give up or the other way
+// round, no more (a larger sum would wait for registers forever; the host refuses a
+// kernel that was not compiled to LAUNCH).  The regularised collision holds the
+// polynomial and the group sums at once: at 64 registers it spills 240 bytes.
+template <bool REGU>
+struct StreamRegs {
+  static constexpr int CTAS = REGU ? 2 : 3, LAUNCH = REGU ? 128 : 80;
+  static constexpr int ADVECT = REGU ? 104 : 96, COLLIDE = REGU ? 152 : 64;
+  static_assert(ADVECT + COLLIDE == 2 * LAUNCH, "");
+};
 constexpr unsigned WAIT_NS = 1000000000u;
 
 template <typename ST>
@@ -761,18 +766,27 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
   }
 }
 
+template <int FROM, int TO>
+__device__ __forceinline__ void role_registers() {
+  if constexpr (TO < FROM)
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(TO));
+  else
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(TO));
+}
+
 template <int ORDER, int LIM, typename ST, bool VEC, bool DIAG, bool REGU, typename Feed>
 __device__ __forceinline__ void stream_roles(const Feed& feed, const StreamSmem<ST>& S,
                                              double& dmass) {
+  using Regs = StreamRegs<REGU>;
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);  // known to be warp-uniform
   if (warp >= 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(COLLIDE_REGS));
+    role_registers<Regs::LAUNCH, Regs::COLLIDE>();
     collide_role<ST, VEC, DIAG, REGU>(feed, S, warp - 4, dmass);
   } else if (warp == 0 || warp == 3) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(ADVECT_REGS));
+    role_registers<Regs::LAUNCH, Regs::ADVECT>();
     advect_role<+1, ORDER, LIM, ST, VEC>(feed, S, warp);
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(ADVECT_REGS));
+    role_registers<Regs::LAUNCH, Regs::ADVECT>();
     advect_role<-1, ORDER, LIM, ST, VEC>(feed, S, warp);
   }
 }
@@ -782,7 +796,7 @@ __device__ __forceinline__ void stream_roles(const Feed& feed, const StreamSmem<
 // are separate instantiations, so that the plain step carries none of their
 // instructions (cold code in the loop body costs instruction fetch).
 template <typename ST, int ORDER, int LIM, bool VEC, bool DIAG, bool REGU>
-__global__ void __launch_bounds__(NT, STREAM_CTAS)
+__global__ void __launch_bounds__(NT, StreamRegs<REGU>::CTAS)
     stream_kernel(const __grid_constant__ StepArgs<float> P, const __grid_constant__ RowMaps maps) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const StreamSmem<ST> S(smem_raw);
@@ -804,7 +818,7 @@ __global__ void __launch_bounds__(NT, STREAM_CTAS)
 // Several lattices advanced by one launch: their work items are concatenated;
 // each lattice brings its own tensor maps.
 template <int ORDER, int LIM, bool REGU>
-__global__ void __launch_bounds__(NT, STREAM_CTAS)
+__global__ void __launch_bounds__(NT, StreamRegs<REGU>::CTAS)
     stream_batch_kernel(const __grid_constant__ BatchArgs<float> B) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const StreamSmem<float> S(smem_raw);
