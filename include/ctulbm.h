@@ -157,7 +157,7 @@ int lbm_step_diag(lbm_handle* h, int64_t n, double threshold, lbm_diag* out);
 
 /* Advance `count` distinct lattices n >= 0 steps together (parameter sweeps,
  * many small jobs).  FP32-shifted lattices with Lx % 4 == 0 and the same
- * scheme and limiter as handles[0] share one fused launch per step, up to 16
+ * scheme and limiter as handles[0] share one fused launch per step, up to 12
  * per launch: their rows are split evenly over one persistent grid, which
  * keeps the GPU full when each lattice alone would not.  Other lattices step
  * on their own.  Every node goes through the same sequence of operations as in
@@ -287,15 +287,17 @@ int lbm_batch_get_info(lbm_batch* b, lbm_batch_info* out);
 
 /* Launch geometry of the handle's fused step kernel (no counterpart in the
  * paper: for tuning, benchmarking and tests).
- *   grid          CTAs of the persistent launch (SMs x resident CTAs at most)
+ *   grid          CTAs of the persistent launch (SMs x resident CTAs at most; a
+ *                 launch that would leave SMs idle has its items handed out in
+ *                 parts of 8 or 4 rows)
  *                 (FP64: of the advection kernel, as the next two)
  *   threads       threads per CTA
  *   smem_bytes    dynamic shared memory per CTA
  *   strips        strips of 56 output columns across x
  *   row_block     rows per work item (work items = strips x row blocks)
- *   tensor_copies 1 when strips away from the periodic x seam stage f^n rows
- *                 with tensor (TMA) copies, 0 when every strip uses per-thread
- *                 16-byte copies (Lx not a multiple of 4, or Lx < 72)
+ *   tensor_copies 1 when f^n rows are staged with tensor (TMA) copies, 0 when
+ *                 they are loaded value by value (Lx not a multiple of 4, or of
+ *                 8 for FP16 storage, or Lx < 72)
  * Returns LBM_ERR_INVALID_ARG for a null argument; the handle is not touched. */
 typedef struct lbm_kernel_info {
   int32_t grid, threads, smem_bytes, strips, row_block, tensor_copies;

@@ -252,14 +252,6 @@ __device__ __forceinline__ void fence_proxy_async() {
 __device__ __forceinline__ void previous_step_done() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
-// A value the compiler does not know: a counter that starts here keeps its loop from
-// being peeled into copies for the first iterations, each of which would have to be
-// fetched once per launch.
-__device__ __forceinline__ int unknown(int v) {
-  int r;
-  asm volatile("mov.b32 %0, %1;\n" : "=r"(r) : "r"(v));
-  return r;
-}
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];\n" ::"l"(map) : "memory");
 }

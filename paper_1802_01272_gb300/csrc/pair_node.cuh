@@ -172,7 +172,7 @@ __device__ __forceinline__ void pair_moments(const StepArgs<typename N::T>& P, L
   using T = typename N::T;
   using V = typename N::V;
   const GroupSums<V> g = group_sums<V, false>(f);
-  dr = add2(g.d[0], add2(g.d[1], add2(g.d[2], g.d[3])));  // the heaviest group last
+  dr = add2(add2(g.d[0], g.d[1]), add2(g.d[2], g.d[3]));
   const V rho = add2(N::dup(P.rho_ref), dr);
   const V ir = N::recip(rho);
   const V lo = N::dup(P.xlo), hi = N::dup(P.xhi);

@@ -191,12 +191,14 @@ struct SingleFeed {
   const StepArgs<float>& P;
   const RowMaps& M;
   int rb, strip, drb, dstrip;  // the next item, and the step of gridDim.x items
+  int blocks;
   __device__ SingleFeed(const StepArgs<float>& p, const RowMaps& m) : P(p), M(m) {
     const unsigned n = (unsigned)P.nstrip;
     rb = (int)(blockIdx.x / n);
     strip = (int)(blockIdx.x - rb * n);
     drb = (int)(gridDim.x / n);
     dstrip = (int)(gridDim.x - drb * n);
+    blocks = (int)((unsigned)(P.Ly + P.row_block - 1) / (unsigned)P.row_block);
   }
   __device__ const StepArgs<float>& args(const Segment&) const { return P; }
   __device__ const CUtensorMap* maps(const Segment&) const { return M.m; }
@@ -204,14 +206,15 @@ struct SingleFeed {
     s.lattice = 0;
     s.strip = strip;
     s.ys = rb * P.row_block;
-    s.ye = min(P.Ly, s.ys + P.row_block);
+    s.ye = s.ys + min(P.row_block, P.Ly - s.ys);
+    const bool more = rb < blocks;
     rb += drb;
     strip += dstrip;
     if (strip >= P.nstrip) {
       strip -= P.nstrip;
       ++rb;
     }
-    return s.ys < P.Ly;
+    return more;
   }
 };
 struct BatchFeed {
@@ -548,7 +551,7 @@ __device__ __forceinline__ void advect_role(Feed feed, const StreamSmem<ST>& S, 
   // this lane's velocities: groups h and h + 2 (equal |xi_x|) of the quadrant
   float* const dst0 = S.fs + (4 * h + q) * REG + col;
   constexpr int D2 = 8 * REG;  // f* ring: group h + 2
-  unsigned g = (unsigned)unknown(0);  // batches so far
+  unsigned g = 0;  // batches so far
   int ring = 0;
   Segment seg;
   while (feed.next(seg)) {
@@ -639,7 +642,7 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
     float dseg = 0.0f;
     int nseg = 0;
 #pragma unroll 1
-    for (int it = unknown(0); it < nit; ++it, ++g) {
+    for (int it = 0; it < nit; ++it, ++g) {
       role_wait(BAR_FULL + (g & 1));
       const int c0 = seg.ys + RPI * (it - WARM);  // first output row of this batch
       // moments of row B - 2 + w (those of a segment's first batch are void: a branch
