@@ -35,8 +35,8 @@
 // barrier and address instructions per node, and replaces three barriers of all
 // warps per batch.  Against one kernel body in which all warps advect, then
 // collide (30 warp instructions per node; now 24): 6144^2 FP32 1.25 -> 1.08
-// ms/step, 2048^2 187 -> 130 us, 1024^2 70 -> 38 us, 1001 x 777 80 -> 39 us, 4096^2
-// FP16 660 -> 511 us.  Measured on the way: two CTAs per SM with 128 registers, as
+// ms/step, 2048^2 187 -> 128 us, 1024^2 70 -> 38 us, 1001 x 777 80 -> 35 us, 4096^2
+// FP16 660 -> 504 us.  Measured on the way: two CTAs per SM with 128 registers, as
 // fast at 1024^2 and 7 % slower at 6144^2; the hand-over by polled mbarriers -3 %;
 // the row loop unrolled by four instead of two -9 % and one copy of the advection
 // per sign quadrant instead of per sign of xi_x -30 % (instruction fetch); seam
