@@ -782,15 +782,17 @@ __device__ __forceinline__ void stream_roles(const Feed& feed, const StreamSmem<
                                              double& dmass) {
   using Regs = StreamRegs<REGU>;
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);  // known to be warp-uniform
+  // setmaxnreg must be one and the same instruction for the four warps of a
+  // warpgroup (warps 0-3, warps 4-7): it comes before any branch inside a group.
   if (warp >= 4) {
     role_registers<Regs::LAUNCH, Regs::COLLIDE>();
     collide_role<ST, VEC, DIAG, REGU>(feed, S, warp - 4, dmass);
-  } else if (warp == 0 || warp == 3) {
-    role_registers<Regs::LAUNCH, Regs::ADVECT>();
-    advect_role<+1, ORDER, LIM, ST, VEC>(feed, S, warp);
   } else {
     role_registers<Regs::LAUNCH, Regs::ADVECT>();
-    advect_role<-1, ORDER, LIM, ST, VEC>(feed, S, warp);
+    if (warp == 0 || warp == 3)
+      advect_role<+1, ORDER, LIM, ST, VEC>(feed, S, warp);
+    else
+      advect_role<-1, ORDER, LIM, ST, VEC>(feed, S, warp);
   }
 }
 

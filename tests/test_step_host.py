@@ -1,0 +1,77 @@
+"""Rules the step kernels must keep that no GPU run shows when they are broken
+(the hardware may still do the expected thing), checked on the CPU: functions of
+the kernels' source, compiled for the host with stand-ins for the device."""
+import os
+import re
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_1802_01272_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return f.read()
+
+
+def _function(text, name):
+    """The definition of the function `name`, from its template line (if any) to its last brace."""
+    m = re.search(r"^(?:template <[^\n]*>\n)?[^\n/]*\b%s\(" % re.escape(name), text, re.M)
+    assert m, name
+    depth = 0
+    for i in range(text.index("{", m.start()), len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[m.start():i + 1]
+    raise AssertionError(name)
+
+
+def _run(tmp_path, code):
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text(code)
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-o", str(exe), str(src)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout
+
+
+@pytest.mark.parametrize("regu", ["false", "true"])
+def test_register_exchange_is_one_instruction_per_warpgroup(tmp_path, regu):
+    """setmaxnreg.aligned: the four warps of a warpgroup execute the same instruction, so
+    every one of them comes to the same place of stream_roles; and each role gets its own."""
+    code = r"""
+#include <cstdio>
+#define __device__
+#define __forceinline__ inline
+struct { int x; } threadIdx;
+int __shfl_sync(unsigned, int v, int) { return v; }
+struct Feed {};
+template <typename ST> struct StreamSmem {};
+template <bool REGU> struct StreamRegs { enum { LAUNCH = 1, ADVECT = 2, COLLIDE = 3 }; };
+int place, amount, role;
+template <int FROM, int TO> void role_registers(int line = __builtin_LINE()) { place = line; amount = TO; }
+template <typename ST, bool V, bool D, bool R, typename F>
+void collide_role(F, const StreamSmem<ST>&, int w, double&) { role = 40 + w; }
+template <int SX, int O, int L, typename ST, bool V, typename F>
+void advect_role(F, const StreamSmem<ST>&, int w) { role = 10 * (SX > 0) + w; }
+""" + _function(_source("step_stream.cuh"), "stream_roles") + r"""
+int main() {
+  StreamSmem<float> S;
+  double m = 0;
+  for (int t = 0; t < 256; t += 32) {
+    threadIdx.x = t;
+    stream_roles<2, 0, float, true, false, REGU>(Feed(), S, m);
+    printf("%d %d %d\n", place, amount, role);
+  }
+}
+""".replace("REGU", regu)
+    warps = [tuple(map(int, s.split())) for s in _run(tmp_path, code).splitlines()]
+    assert len(warps) == 8
+    assert len({w[0] for w in warps[:4]}) == 1 and len({w[0] for w in warps[4:]}) == 1, warps
+    assert [w[1] for w in warps] == [2] * 4 + [3] * 4
+    # quadrants (+,+), (-,+), (-,-), (+,-): the sign of xi_x of each advect warp
+    assert [w[2] for w in warps] == [10, 1, 2, 13, 40, 41, 42, 43]
