@@ -123,20 +123,26 @@ __device__ __forceinline__ bool bar_try_wait(unsigned bar, unsigned parity) {
 // Waits for a phase of `bar`, at most WAIT_NS; false if it was not seen to
 // complete.  A timeout sets error bit 1 and the warp's abort flag, after which
 // none of its waits waits (the results are void): every role runs to its end.
+// Warp-collective, and the whole warp gets one answer: a lane's clock may pass the
+// limit while its neighbours see the phase complete, and warp-wide instructions
+// follow under the answer.
 __device__ __forceinline__ bool stream_wait(unsigned bar, unsigned parity, int* abort,
                                             unsigned* err) {
-  if (bar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
+  bool ok = bar_try_wait(bar, parity);
+  if (!ok) {
+    const unsigned long long t0 = global_ns();
 #pragma unroll 1
-  for (;;) {
-    if (bar_try_wait(bar, parity)) return true;
-    if (*reinterpret_cast<volatile int*>(abort)) return false;
-    if (global_ns() - t0 > WAIT_NS) {
-      *reinterpret_cast<volatile int*>(abort) = 1;
-      atomicOr(err, 2u);
-      return false;
+    for (;;) {
+      ok = bar_try_wait(bar, parity);
+      if (ok || *reinterpret_cast<volatile int*>(abort)) break;
+      if (global_ns() - t0 > WAIT_NS) {
+        *reinterpret_cast<volatile int*>(abort) = 1;
+        atomicOr(err, 2u);
+        break;
+      }
     }
   }
+  return __all_sync(0xffffffffu, ok);
 }
 // One lane of the (converged) warp: a predicate the compiler knows to hold for
 // a single thread, so that a tensor copy under it needs no loop over lanes.

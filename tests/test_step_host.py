@@ -75,3 +75,66 @@ int main() {
     assert [w[1] for w in warps] == [2] * 4 + [3] * 4
     # quadrants (+,+), (-,+), (-,-), (+,-): the sign of xi_x of each advect warp
     assert [w[2] for w in warps] == [10, 1, 2, 13, 40, 41, 42, 43]
+
+
+def test_wait_gives_a_warp_one_answer(tmp_path):
+    """stream_wait on 32 threads as the lanes of a warp, each with its own clock and its own view
+    of the barrier: whatever mix of completions and timeouts the lanes see, all return the same;
+    a timeout is reported, and a warp that saw the phase complete in every lane goes on."""
+    code = r"""
+#include <atomic>
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include <pthread.h>
+#define __device__
+#define __forceinline__ inline
+constexpr unsigned WAIT_NS = 1000000000u;
+int scenario;
+thread_local int lane, polls;
+thread_local unsigned long long clock_ns;
+std::atomic<int> seen;
+std::atomic<unsigned> errors;
+pthread_barrier_t gate;
+// 0: complete at once; 1: complete later; 2: never; 3: lane 7's clock runs out, the others then
+// see the phase complete; 4: lane 0 sees it at the first poll, the others never
+bool bar_try_wait(unsigned, unsigned) {
+  ++polls;
+  switch (scenario) {
+    case 0: return true;
+    case 1: return polls > 5;
+    case 2: return false;
+    case 3:
+      if (lane != 7) while (!errors.load()) std::this_thread::yield();
+      return lane != 7;
+    default: return lane == 0;
+  }
+}
+unsigned long long global_ns() { return clock_ns += (scenario == 3 && lane == 7 ? 600000000ull : 100000000ull); }
+void atomicOr(unsigned*, unsigned v) { errors |= v; }
+bool __all_sync(unsigned, bool v) {
+  if (v) ++seen;
+  pthread_barrier_wait(&gate);
+  return seen.load() == 32;
+}
+""" + _function(_source("step_stream.cuh"), "stream_wait") + r"""
+int main() {
+  for (scenario = 0; scenario < 5; ++scenario) {
+    int abort = 0;
+    unsigned err = 0;
+    bool got[32];
+    seen = 0;
+    errors = 0;
+    pthread_barrier_init(&gate, nullptr, 32);
+    std::vector<std::thread> warp;
+    for (int l = 0; l < 32; ++l)
+      warp.emplace_back([&, l] { lane = l; got[l] = stream_wait(0, 0, &abort, &err); });
+    for (auto& t : warp) t.join();
+    int n = 0;
+    for (bool g : got) n += g;
+    printf("%d %d %u\n", n, abort, errors.load());
+  }
+}
+"""
+    got = [tuple(map(int, s.split())) for s in _run(tmp_path, code).splitlines()]
+    assert got == [(32, 0, 0), (32, 0, 0), (0, 1, 2), (0, 1, 2), (0, 1, 2)], got
