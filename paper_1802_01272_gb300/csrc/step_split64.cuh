@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(NT, 2)
           if (P.walls && (unsigned)row >= (unsigned)Ly)  // wall ghost rows
             in[i] = row < 0 ? v.gbot : v.gtop;
           else
-            in[i] = __ldg(col + (long long)wrap_row(row, Ly) * Lx);
+            in[i] = col[(long long)wrap_row(row, Ly) * Lx];
         }
       }
       __syncwarp();  // slot (b + 2) % 3 was read with batch b - 1
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(C64_NT)
     } else {
       const double* src = fin + (long long)wrap_row(row, Ly) * Lx + x;
 #pragma unroll
-      for (int k = 0; k < 16; ++k) f[k] = __ldg(src + k * pl);
+      for (int k = 0; k < 16; ++k) f[k] = src[k * pl];
     }
     double d[4];
 #pragma unroll
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(C64_NT)
     const double* src = fin + (long long)y * Lx + x;
     double f[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) f[k] = __ldg(src + k * pl);
+    for (int k = 0; k < 16; ++k) f[k] = src[k * pl];
     const auto load = [&](int k) { return f[k]; };
     const double *ph[5], *dq[5];
 #pragma unroll

@@ -449,8 +449,8 @@ static __device__ __forceinline__ void stage_values(ST* dst, unsigned bar, const
       ST v[8];
 #pragma unroll
       for (int grp = 0; grp < 4; ++grp) {
-        v[2 * grp] = __ldg(pa + 4 * grp * plane);
-        v[2 * grp + 1] = __ldg(pb + 4 * grp * plane);
+        v[2 * grp] = pa[4 * grp * plane];
+        v[2 * grp + 1] = pb[4 * grp * plane];
       }
 #pragma unroll
       for (int grp = 0; grp < 4; ++grp) {

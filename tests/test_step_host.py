@@ -138,3 +138,13 @@ int main() {
 """
     got = [tuple(map(int, s.split())) for s in _run(tmp_path, code).splitlines()]
     assert got == [(32, 0, 0), (32, 0, 0), (0, 1, 2), (0, 1, 2), (0, 1, 2)], got
+
+
+@pytest.mark.parametrize("name", ["lbm_kernels.cuh", "pair_node.cuh", "step_stream.cuh",
+                                  "step_split64.cuh"])
+def test_dependently_launched_kernels_read_coherently(name):
+    """A step's kernel is on the device while the one before it still writes the buffers it will
+    read.  A non-coherent load is only defined on data that nothing writes during the kernel, and
+    may be moved before the wait for the previous kernel: none in these sources."""
+    code = re.sub(r"//[^\n]*", "", _source(name))
+    assert re.findall(r"__ldg\b|ld\.global\.(?:\w+\.)*nc\b|__restrict__", code) == []
