@@ -203,7 +203,15 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
   a.pg = (T)(3.0 - 2.0 * p.T);
   a.p20 = (T)(om * ps);
   a.p30 = (T)(-2.0 * om / 3.0);
-  for (int i = 0; i < 3; ++i) a.w[i] = (T)h->w[4 * i + (i == 2 ? 4 : 0)];
+  a.om2 = (T)(0.5 * om);
+  a.om6 = (T)(om / 6.0);
+  for (int i = 0; i < 3; ++i) {
+    const int k = 4 * i + (i == 2 ? 4 : 0);
+    a.w[i] = (T)h->w[k];
+    const double x2 = h->xi[k][0] * h->xi[k][0] + h->xi[k][1] * h->xi[k][1];
+    const double A = (p.T - 1.0) * (x2 - 2.0) / 2.0, B = (p.T - 1.0) * (x2 - 4.0) / 2.0;
+    a.cls[i] = {(float)(om * A), (float)A, (float)(om * B)};
+  }
   double gb[16], gt[16];
   const double uw = p.shear_rate * p.Ly * p.ds / 2.0;
   feq_host(p, h->xi, h->w, p.rho_ext, -uw, 0.0, gb);
@@ -212,7 +220,7 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
     const double x = h->xi[k][0], y = h->xi[k][1];
     const double ax = std::fabs(x), ay = std::fabs(y);
     const double cx = lam * ax, cy = lam * ay;
-    const double hx = 0.5 * ax * (1.0 - cx);
+    const double hx = 0.5 * ax * (1.0 - cx), hy = 0.5 * ay * (1.0 - cy);
     VelConst<T>& v = a.v[k];
     v.xi_x = (T)x;
     v.xi_y = (T)y;
@@ -228,6 +236,8 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
     v.ax = (T)(2.0 * lam * hx);
     v.qy0 = (T)((1.0 - cy) * (1.0 - cx));
     v.qy1 = (T)((1.0 - cy) * cx);
+    v.by0 = (T)(-2.0 * lam * hy * (1.0 - cx));
+    v.by1 = (T)(-2.0 * lam * hy * cx);
     v.gbot = (T)(gb[k] - h->w[k] * rr);
     v.gtop = (T)(gt[k] - h->w[k] * rr);
   }

@@ -56,6 +56,11 @@ struct __align__(W * sizeof(S)) Run {
   S v[W];
 };
 
+// A product that stays one (the compiler would contract it with a sum, and not in the
+// same way in each instantiation: the results must not depend on which one runs).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // Eq. (herfeq) with the storage shift w_k rho_ref removed:
 // f^eq - w rho_ref = w [ (rho - rho_ref) + rho (P_k - 1) ],
 // P_k - 1 = xi.u + [(xi.u)^2 - u^2 + (T-1)(xi^2-2)]/2 + xi.u [(xi.u)^2 - 3u^2 + 3(T-1)(xi^2-4)]/6
@@ -79,18 +84,19 @@ __global__ void init_feq_kernel(const AuxArgs a, S* f, const double* rho, const 
     dr[e] = (T)(in[0].v[e] - a.rho_ref);
     u[e] = (T)in[1].v[e];
     w[e] = (T)in[2].v[e];
-    u2[e] = u[e] * u[e] + w[e] * w[e];
+    u2[e] = fma(u[e], u[e], mul_rn(w[e], w[e]));
   }
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const T x2 = v.x[k] * v.x[k] + v.y[k] * v.y[k];
+    const T x2 = fma(v.y[k], v.y[k], mul_rn(v.x[k], v.x[k]));
     Run<S, W> o;
 #pragma unroll
     for (int e = 0; e < W; ++e) {
-      const T cu = v.x[k] * u[e] + v.y[k] * w[e];
-      const T pm1 = cu + T(0.5) * (cu * cu - u2[e] + Tm1 * (x2 - T(2))) +
-                    cu / T(6) * (cu * cu - T(3) * u2[e] + T(3) * Tm1 * (x2 - T(4)));
-      o.v[e] = to_store<S, T>(v.w[k] * (dr[e] + r[e] * pm1));
+      const T cu = fma(v.x[k], u[e], mul_rn(v.y[k], w[e])), c2 = mul_rn(cu, cu);
+      const T a2 = fma(Tm1, x2 - T(2), c2 - u2[e]);
+      const T a3 = fma(T(3) * Tm1, x2 - T(4), fma(T(-3), u2[e], c2));
+      const T pm1 = fma(cu / T(6), a3, fma(T(0.5), a2, cu));
+      o.v[e] = to_store<S, T>(v.w[k] * fma(r[e], pm1, dr[e]));
     }
     *reinterpret_cast<Run<S, W>*>(f + k * a.plane + q) = o;
   }
@@ -114,25 +120,18 @@ __global__ void get_f_kernel(const AuxArgs a, const S* f, double* dst) {
     dst[k * a.plane + q] = (double)from_store<S, T>(f[k * a.plane + q]) + a.w[k] * a.rho_ref;
 }
 
-// rho - rho_ref = sum_k f_k and rho u = sum_k f_k xi_k of a node's stored (shifted) f;
-// velocity order k = 4 group + sign, signs (+,+), (-,+), (-,-), (+,-).  The groups are
-// summed from the lightest to the heaviest: a vapour node's deviations are as large
-// as the liquid's density, and each sum near the total costs a rounding of it.
+// rho - rho_ref = sum_k f_k and rho u = sum_k f_k xi_k of a node's stored (shifted) f, in
+// velocity order (the order is part of the results: the same f gives the same moments).
 template <typename T>
 __device__ __forceinline__ void node_moments(const AuxArgs& a, const Vel<T>& v, const T (&f)[16],
                                              T& drho, T& mx, T& my) {
-  T d[4], sx[4], sy[4];
+  drho = mx = my = T(0);
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    const T p = f[4 * g] + f[4 * g + 2], q = f[4 * g + 1] + f[4 * g + 3];
-    const T m = f[4 * g] - f[4 * g + 2], n = f[4 * g + 1] - f[4 * g + 3];
-    d[g] = p + q;
-    sx[g] = m - n;
-    sy[g] = m + n;
+  for (int k = 0; k < 16; ++k) {
+    drho += f[k];
+    mx += f[k] * v.x[k];
+    my += f[k] * v.y[k];
   }
-  drho = d[0] + ((d[1] + d[2]) + d[3]);
-  mx = v.x[0] * (sx[0] + sx[2]) + v.x[4] * (sx[1] + sx[3]);
-  my = v.y[0] * (sy[0] + sy[1]) + v.y[8] * (sy[2] + sy[3]);
 }
 template <typename S, typename T>
 __device__ __forceinline__ void node_moments_at(const AuxArgs& a, const Vel<T>& v, const S* f,

@@ -35,8 +35,15 @@ struct VelConst {
   T xi_x, xi_y, w;
   T cx, cy;                 // Courant numbers |xi_x| dt/ds, |xi_y| dt/ds
   T ax;                     // lam |xi_x| (1 - cx): weight of the x-difference of half-limited S^x
-  T qy0, qy1;               // (1 - cy) (1 - cx), (1 - cy) cx: weights of the S^y terms per unit of cy
+  T qy0, qy1;               // FP64: (1 - cy) (1 - cx), (1 - cy) cx: weights of the S^y terms per unit of cy
+  T by0, by1;               // FP32: -cy (1 - cy) (1 - cx), -cy (1 - cy) cx: weights of the dS^y terms
   T gbot, gtop;             // wall ghost-row values (storage variable)
+};
+
+// Per-class constants of the FP32 collision (velocity groups with the same xi^2):
+// w A, A, w B with A = (T - 1)(xi^2 - 2)/2, B = (T - 1)(xi^2 - 4)/2, w = dt/tau.
+struct ClassConst {
+  float omA, A, omB;
 };
 
 template <typename T>
@@ -72,6 +79,8 @@ struct StepArgs {
   // 3 - 2 T, w s, -2 w / 3
   T ps, p00, p10, pg, p20, p30;
   T w[3];                   // weights of the groups (lo,lo), (hi,lo) = (lo,hi), (hi,hi)
+  T om2, om6;               // w/2, w/6
+  ClassConst cls[3];        // of the same groups
   VelConst<T> v[16];
 };
 
@@ -167,10 +176,21 @@ __device__ __forceinline__ double shfl_dn1(double v) { return __shfl_down_sync(0
 // ------------------------------------------------------- pairs of values
 // Two neighbouring columns or nodes as one value: in FP32 every operation on
 // whole pairs is one packed FP32x2 instruction (sm_100+, round to nearest),
-// which issues once for two lanes' worth of work.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+// which issues once for two lanes' worth of work.  A product that only feeds a sum
+// is written as one fma2: left apart, the two are contracted in some kernels and
+// not in others (also where both are marked .rn), and a node would step
+// differently in each.
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// (a sum as an intrinsic: 6144^2 1111 us per step against 1107, 4096^2 FP16 537 against 530)
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<const unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<const unsigned long long*>(&b)));
+  return *reinterpret_cast<const float2*>(&r);
+}
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   unsigned long long r;
   asm("sub.rn.f32x2 %0, %1, %2;"

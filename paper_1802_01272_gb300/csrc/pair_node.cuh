@@ -32,7 +32,7 @@ struct NodeConst {
   V lo, hi, nlo, nhi, lo2, hi2;
   V w[3];
   __device__ explicit NodeConst(const StepArgs<typename N::T>& P)
-      : gw1(N::dup(P.gw1)), gw2(N::dup(P.gw2)), gw3(N::dup(P.gw3)), gw4(N::dup(P.gw4)), om(N::dup(P.omega)),
+      : gw1(N::dup(P.gw1)), gw2(N::dup(P.gw2)), gw3(N::dup(-P.gw3)), gw4(N::dup(-P.gw4)), om(N::dup(P.omega)),
         ps(N::dup(P.ps)), p00(N::dup(P.p00)), p10(N::dup(P.p10)), pg(N::dup(P.pg)), p20(N::dup(P.p20)),
         p30(N::dup(P.p30)), lo(N::dup(P.xlo)), hi(N::dup(P.xhi)), nlo(N::dup(-P.xlo)), nhi(N::dup(-P.xhi)),
         lo2(N::dup(P.lo2)), hi2(N::dup(P.hi2)) {
@@ -53,10 +53,6 @@ __device__ __forceinline__ Row6<V> row6(const T* p) {
           *reinterpret_cast<const V*>(p + 2)};
 }
 template <typename V>
-__device__ __forceinline__ Row6<V> add_rows(const Row6<V>& a, const Row6<V>& b) {
-  return {add2(a.l, b.l), add2(a.m, b.m), add2(a.r, b.r)};
-}
-template <typename V>
 __device__ __forceinline__ Row6<V> sub_rows(const Row6<V>& a, const Row6<V>& b) {
   return {sub2(a.l, b.l), sub2(a.m, b.m), sub2(a.r, b.r)};
 }
@@ -68,8 +64,8 @@ __device__ __forceinline__ Row6<V> sub_rows(const Row6<V>& a, const Row6<V>& b) 
 //  * kappa grad(lap rho*): D_h of the isotropic 9-point Laplacian, the two
 //    composed into one 5x5 stencil on rho* - rho_ref (the Laplacian of a
 //    constant vanishes).
-// Both stencils are even across the derivative's direction, so rows are added
-// (for d/dx) or subtracted (for d/dy) first and the sums shared by the pair.
+// Every sum is of differences across the node (the density's large constant part
+// cancels before anything is added), from the nearest to the farthest.
 template <typename N>
 __device__ __forceinline__ void pair_force(const NodeConst<N>& C, const typename N::T* const (&ph)[5],
                                            const typename N::T* const (&dq)[5], typename N::V ir,
@@ -80,36 +76,30 @@ __device__ __forceinline__ void pair_force(const NodeConst<N>& C, const typename
   using V = typename N::V;
   V px, py, lx, ly;
   if constexpr (N::W == 2) {
+  // rows c - 2 .. c + 2: differences one and two columns apart, and between rows
+  const auto d1x = [](const Row6<V>& r) { return N::make(r.m.y - r.l.y, r.r.x - r.m.x); };
+  const auto d2x = [](const Row6<V>& r) { return sub2(r.r, r.l); };
+  const auto sum1 = [](const Row6<V>& d) { return N::make(d.m.y + d.l.y, d.r.x + d.m.x); };
+  const auto sum2 = [](const Row6<V>& d) { return add2(d.r, d.l); };
   {
     const Row6<V> t0 = row6<V>(ph[2]), up = row6<V>(ph[3]), dn = row6<V>(ph[1]);
-    const Row6<V> t1 = add_rows(up, dn), d1 = sub_rows(up, dn);
     const Row6<V> up2 = row6<V>(ph[4]), dn2 = row6<V>(ph[0]);
-    const Row6<V> d2 = sub_rows(up2, dn2);
-    const V t2l = add2(up2.l, dn2.l), t2r = add2(up2.r, dn2.r);
-    const V w1 = C.gw1, w2 = C.gw2, w3 = C.gw3, w4 = C.gw4;
-    const V al = fma2(w1, t0.l, mul2(w2, t1.l)), am = fma2(w1, t0.m, mul2(w2, t1.m)),
-            ar = fma2(w1, t0.r, mul2(w2, t1.r));
-    const V bl = fma2(w3, t0.l, mul2(w4, t2l)), br = fma2(w3, t0.r, mul2(w4, t2r));
-    px = sub2(N::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
-    const V e1 = N::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d2.r, d2.l);
-    py = sub2(fma2(w1, d1.m, mul2(w2, e1)), fma2(w3, d2.m, mul2(w4, e2)));
+    const V w1 = C.gw1, w2 = C.gw2, w3 = C.gw3, w4 = C.gw4;  // (w3 and w4 negated)
+    px = fma2(w1, d1x(t0), fma2(w2, add2(d1x(up), d1x(dn)),
+              fma2(w3, d2x(t0), mul2(w4, add2(d2x(up2), d2x(dn2))))));
+    const Row6<V> d1 = sub_rows(up, dn), d2 = sub_rows(up2, dn2);
+    py = fma2(w1, d1.m, fma2(w2, sum1(d1), fma2(w3, d2.m, mul2(w4, sum2(d2)))));
   }
   {
     const Row6<V> t0 = row6<V>(dq[2]), up = row6<V>(dq[3]), dn = row6<V>(dq[1]);
     drho = t0.m;
-    const Row6<V> t1 = add_rows(up, dn), d1 = sub_rows(up, dn);
     const Row6<V> up2 = row6<V>(dq[4]), dn2 = row6<V>(dq[0]);
-    const Row6<V> t2 = add_rows(up2, dn2), d2 = sub_rows(up2, dn2);
     const V k0 = C.kw[0], k1 = C.kw[1], k2 = C.kw[2], k3 = C.kw[3], k4 = C.kw[4], k5 = C.kw[5];
-    const V al = fma2(k0, t0.l, fma2(k1, t1.l, mul2(k2, t2.l)));
-    const V am = fma2(k0, t0.m, fma2(k1, t1.m, mul2(k2, t2.m)));
-    const V ar = fma2(k0, t0.r, fma2(k1, t1.r, mul2(k2, t2.r)));
-    const V bl = fma2(k3, t0.l, fma2(k4, t1.l, mul2(k5, t2.l)));
-    const V br = fma2(k3, t0.r, fma2(k4, t1.r, mul2(k5, t2.r)));
-    lx = add2(N::make(am.y - al.y, ar.x - am.x), sub2(br, bl));
-    const V e1 = N::make(d1.m.y + d1.l.y, d1.r.x + d1.m.x), e2 = add2(d1.r, d1.l);
-    const V h1 = N::make(d2.m.y + d2.l.y, d2.r.x + d2.m.x), h2 = add2(d2.r, d2.l);
-    ly = fma2(k0, d1.m, fma2(k1, e1, fma2(k2, e2, fma2(k3, d2.m, fma2(k4, h1, mul2(k5, h2))))));
+    lx = fma2(k0, d1x(t0), fma2(k1, add2(d1x(up), d1x(dn)), fma2(k2, add2(d1x(up2), d1x(dn2)),
+         fma2(k3, d2x(t0), fma2(k4, add2(d2x(up), d2x(dn)), mul2(k5, add2(d2x(up2), d2x(dn2))))))));
+    const Row6<V> d1 = sub_rows(up, dn), d2 = sub_rows(up2, dn2);
+    ly = fma2(k0, d1.m, fma2(k1, sum1(d1), fma2(k2, sum2(d1),
+         fma2(k3, d2.m, fma2(k4, sum1(d2), mul2(k5, sum2(d2)))))));
   }
   } else {
     // one node: columns c - 2 .. c + 2 of five rows
@@ -119,11 +109,11 @@ __device__ __forceinline__ void pair_force(const NodeConst<N>& C, const typename
       const T x1 = diff(p[2][1], p[2][-1]), x2 = diff(p[2][2], p[2][-2]);
       const T xd1 = diff(p[3][1] + p[1][1], p[3][-1] + p[1][-1]);
       const T xd2 = diff(p[4][2] + p[0][2], p[4][-2] + p[0][-2]);
-      px = fma(C.gw1, x1, C.gw2 * xd1) - fma(C.gw3, x2, C.gw4 * xd2);
+      px = fma(C.gw1, x1, C.gw2 * xd1) + fma(C.gw3, x2, C.gw4 * xd2);
       const T y1 = diff(p[3][0], p[1][0]), y2 = diff(p[4][0], p[0][0]);
       const T yd1 = diff(p[3][1], p[1][1]) + diff(p[3][-1], p[1][-1]);
       const T yd2 = diff(p[4][2], p[0][2]) + diff(p[4][-2], p[0][-2]);
-      py = fma(C.gw1, y1, C.gw2 * yd1) - fma(C.gw3, y2, C.gw4 * yd2);
+      py = fma(C.gw1, y1, C.gw2 * yd1) + fma(C.gw3, y2, C.gw4 * yd2);
     }
     {
       const T* const(&p)[5] = dq;
@@ -330,6 +320,53 @@ __device__ __forceinline__ void regularised_poly(const StepArgs<typename N::T>& 
   join(p.c21, r.c21);
   join(p.c12, r.c12);
   join(p.c03, r.c03);
+}
+
+// The plain collision in FP32, by velocity groups: with cu = xi.u, D = dt xi.g,
+// w = dt/tau, A = (T - 1)(xi^2 - 2)/2, B = (T - 1)(xi^2 - 4)/2, e = 1 - u^2/2,
+//   [w f^eq + dt F_k - w w_k rho_ref] / (w_k rho) = E + O,
+//   E = w/2 cu^2 + D cu + w (rho - rho_ref)/rho + w (e - 1) - dt g.u + w A,
+//   O = cu [w/6 cu^2 + w e - dt g.u + w B] + D [cu^2/2 + e - T + 1 + A],
+// and the opposite velocity is E - O.  Each operation and its order is part of the
+// result: an FP32 step returns the same bits in every kernel, whatever the launch,
+// and FP16 storage would turn another order into flipped roundings of f.  As the
+// polynomial below it is a quarter fewer instructions for the pair (6144^2 1076
+// us per step against 1107, 4096^2 FP16 504 against 530), but the density at a
+// vapour node then drifts from the FP64 step's by 1.4e-6 of its value in 100
+// steps where this form gives 6e-8 (sheared bubble, 1024 x 512).
+template <typename Load, typename Put>
+__device__ __forceinline__ void group_collide(const StepArgs<float>& P, const NodeConst<Pair32>& C, Load f,
+                                              Put put, float2 drho, float2 rho, float2 ir, float2 u,
+                                              float2 v, float2 g, float2 h) {
+  const float2 half = dup2(0.5f), one = dup2(1.0f), s1 = dup2(P.one_m_omega);
+  const float2 e = fma2(dup2(-0.5f), fma2(u, u, mul2(v, v)), one);
+  const float2 gu = fma2(g, u, mul2(h, v));
+  const float2 p0 = sub2(fma2(C.om, sub2(e, one), mul2(mul2(C.om, drho), ir)), gu);
+  const float2 p1 = add2(sub2(e, dup2(P.Tt)), one);
+  const float2 p2 = fma2(C.om, e, make_float2(-gu.x, -gu.y));
+#pragma unroll
+  for (int iy = 0; iy < 2; ++iy) {
+    const float2 Y = iy ? C.hi : C.lo;
+#pragma unroll
+    for (int ix = 0; ix < 2; ++ix) {
+      const float2 X = ix ? C.hi : C.lo, xu = mul2(X, u), xg = mul2(X, g);
+      const float2 nxu = make_float2(-xu.x, -xu.y), nxg = make_float2(-xg.x, -xg.y);
+      const ClassConst& cl = P.cls[ix + iy];
+      const float2 P0 = add2(p0, dup2(cl.omA)), P1 = add2(p1, dup2(cl.A)), K = add2(p2, dup2(cl.omB));
+      const float2 sw = mul2(C.w[ix + iy], rho), nsw = mul2(make_float2(-C.w[ix + iy].x, -C.w[ix + iy].y), rho);
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const int k = 4 * (2 * iy + ix) + m;  // signs in a group: (+,+), (-,+), (-,-), (+,-)
+        const float2 cu = fma2(Y, v, m ? nxu : xu), D = fma2(Y, h, m ? nxg : xg);
+        const float2 c2 = mul2(cu, cu);
+        const float2 E = fma2(c2, dup2(P.om2), fma2(cu, D, P0));
+        const float2 O = fma2(cu, fma2(c2, dup2(P.om6), K), mul2(D, fma2(c2, half, P1)));
+        const float2 Q = mul2(sw, E);
+        put(k, fma2(s1, f(k), fma2(sw, O, Q)));
+        put(k + 2, fma2(s1, f(k + 2), fma2(nsw, O, Q)));
+      }
+    }
+  }
 }
 
 // Collision of two nodes: f(k) loads f*_k, put(k, value) receives f^{n+1}_k.

@@ -247,23 +247,21 @@ struct BatchFeed {
 
 // ------------------------------------------------------------- advection
 // Row history of four columns (two pairs) of one velocity.  Z is the x part of
-// the update, Z = f - c_x (f - f(i - s_x)) - ax dS^x.  With the S^y terms
-// collected into Q = Z -+ [(1 - c_x) S^y(i) + c_x S^y(i - s_x)] (1 - c_y) at the
-// face downwind of row j (S^y(j + 1), upper sign) for s_y > 0, at its upper face
-// (S^y(j), lower sign) for s_y < 0, the update of row j is
-//   s_y > 0: Z(j) + c_y (Q(j - 1) - Q(j)),   s_y < 0: Z(j) - c_y (Q(j) - Q(j + 1))
-// (Sec. II C 2 collected per node); a uniform state is kept exactly.  When row n
-// arrives Q(n - 1) is known for both signs, so row n - 2 is emitted as
-// W + cm [Q(n - 2) - Q(n - 1)], W = Z(n - 2) + cp [Q(n - 3) - Q(n - 2)], with one
-// of (cp, cm) = (c_y, 0), (0, -c_y): the sign of xi_y is data, and the four
-// quadrants run two copies of the code instead of four (the instruction cache
-// holds the roles' loops; four copies cost a third of the speed).
+// the update, Z = f - c_x (f - f(i - s_x)) - ax dS^x; the update of row j is
+//   Z(j) + c_y (Z(j - s_y) - Z(j)) + by0 dS^y(i) + by1 dS^y(i - s_x),
+// dS^y = S^y(j + 1) - S^y(j) (Sec. II C 2 collected per node); a uniform state is
+// kept exactly.  When row n arrives, S^y is known up to row n for s_y > 0 and row
+// n - 1 for s_y < 0, which makes row n - 1 or n - 2 complete: a warp with s_y > 0
+// stages one row behind, so that all emit the same rows.  The sign of xi_y is data
+// (cy carries it), and the four quadrants run two copies of the code instead of
+// four (the instruction cache holds the roles' loops; four copies cost a third of
+// the speed).
 struct StreamState {
-  float2 F[2], Ry[2], Z1[2];  // f, R^y and Z of the row before
-  float2 Q1[2], W[2];         // Q(n - 2); W as above
+  float2 F[2], Ry[2], Sy[2];  // f, R^y and S^y of the row before
+  float2 Z1[2], Z2[2];        // Z of the two rows before
 };
 struct StreamConst {
-  float2 cp, cm, b0;  // as above; weights of S^y(i) and (b1) S^y(i - s_x) in Q, signed
+  float2 cy, b0;  // s_y c_y; weights of dS^y(i) and (b1) dS^y(i - s_x)
   float b1;
 };
 struct StreamConstX {
@@ -271,7 +269,7 @@ struct StreamConstX {
 };
 
 // One staged row n of a velocity with s_x = SX, own columns (0, 1) in
-// B0 and (2, 3) in B1; out receives the advected row n - 2.  All lanes of a
+// B0 and (2, 3) in B1; out receives the advected row n - 1 (sy) or n - 2.  All lanes of a
 // warp call it together.  The two edge lanes of a velocity's 16 get no useful
 // neighbours: region columns 0, 1, 62, 63 come out void and feed no output.
 template <int SX, int ORDER, int LIM>
@@ -298,8 +296,7 @@ __device__ __forceinline__ void stream_row(StreamState& s, float2 B0, float2 B1,
       S4 = shfl_dn1(S0);
     }
   } else {
-    // columns 4, 5; S^x(i) from R(i) and R(i+1), quarter sum (f(i+1) - f(i-1))/4,
-    // taken at columns 1 .. 4 so that the sums are of whole pairs
+    // columns 4, 5; S^x(i) from R(i) and R(i+1), taken at columns 1 .. 4
     const float Ex = shfl_dn1(B0.x);
     const float R1 = B0.y - B0.x, R2 = B1.x - B0.y, R3 = B1.y - B1.x, R4 = Ex - B1.y;
     Z[0] = fma2(c.ncx, make_float2(R1, R2), B0);
@@ -307,7 +304,8 @@ __device__ __forceinline__ void stream_row(StreamState& s, float2 B0, float2 B1,
     if constexpr (ORDER == 2) {
       const float Ey = shfl_dn1(B0.y);
       const float R5 = Ey - Ex;
-      const float2 h12 = mul2(c.q, sub2(B1, B0)), h34 = mul2(c.q, sub2(make_float2(Ex, Ey), B1));
+      const float2 h12 = mul2(c.q, make_float2(R1 + R2, R2 + R3));
+      const float2 h34 = mul2(c.q, make_float2(R3 + R4, R4 + R5));
       S1 = mc_half<LIM>(R1, R2, h12.x);
       S2 = mc_half<LIM>(R2, R3, h12.y);
       S3 = mc_half<LIM>(R3, R4, h34.x);
@@ -320,10 +318,15 @@ __device__ __forceinline__ void stream_row(StreamState& s, float2 B0, float2 B1,
     Z[1] = fma2(c.nax, make_float2(S3 - S2, S4 - S3), Z[1]);
   }
 
-  float2 Q[2] = {s.Z1[0], s.Z1[1]};
   const float2 B[2] = {B0, B1};
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    // cy carries the sign of s_y: Z(j) + c_y (Z(j - s_y) - Z(j)) for either
+    const float2 D = sub2(s.Z2[m], s.Z1[m]);
+    out[m] = fma2(k.cy, D, sy ? s.Z1[m] : s.Z2[m]);
+  }
   if constexpr (ORDER == 2) {
-    float2 Sy[2];
+    float2 dS[2];
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
       const float2 Ry = sub2(B[m], s.F[m]);
@@ -331,36 +334,34 @@ __device__ __forceinline__ void stream_row(StreamState& s, float2 B0, float2 B1,
       // s_y > 0: S^y(n), from R^y(n) with the upwind jump R^y(n - 1); s_y < 0:
       // S^y(n - 1), from R^y(n - 1) with R^y(n) (the MC form is symmetric in the two)
       const float2 a = LIM == 0 || sy ? Ry : s.Ry[m], b = LIM == 0 || sy ? s.Ry[m] : Ry;
-      Sy[m] = make_float2(mc_half<LIM>(a.x, b.x, h.x), mc_half<LIM>(a.y, b.y, h.y));
+      const float2 Sy = make_float2(mc_half<LIM>(a.x, b.x, h.x), mc_half<LIM>(a.y, b.y, h.y));
+      dS[m] = sub2(Sy, s.Sy[m]);
       s.Ry[m] = Ry;
+      s.Sy[m] = Sy;
     }
-    // S^y one column upwind in x
-    const float e = SX > 0 ? shfl_up1(Sy[1].y) : shfl_dn1(Sy[0].x);
-    const float u[4] = {SX > 0 ? e : Sy[0].y, SX > 0 ? Sy[0].x : Sy[1].x,
-                        SX > 0 ? Sy[0].y : Sy[1].y, SX > 0 ? Sy[1].x : e};
+    // dS^y one column upwind in x
+    const float e = SX > 0 ? shfl_up1(dS[1].y) : shfl_dn1(dS[0].x);
+    const float u[4] = {SX > 0 ? e : dS[0].y, SX > 0 ? dS[0].x : dS[1].x,
+                        SX > 0 ? dS[0].y : dS[1].y, SX > 0 ? dS[1].x : e};
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-      const float2 t = fma2(k.b0, Sy[m], Q[m]);
-      Q[m] = make_float2(fmaf(k.b1, u[2 * m], t.x), fmaf(k.b1, u[2 * m + 1], t.y));
+      const float2 t = fma2(k.b0, dS[m], out[m]);
+      out[m] = make_float2(fmaf(k.b1, u[2 * m], t.x), fmaf(k.b1, u[2 * m + 1], t.y));
     }
   }
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
-    const float2 D = sub2(s.Q1[m], Q[m]);
-    out[m] = fma2(k.cm, D, s.W[m]);
-    s.W[m] = fma2(k.cp, D, s.Z1[m]);
     s.F[m] = B[m];
+    s.Z2[m] = s.Z1[m];
     s.Z1[m] = Z[m];
-    s.Q1[m] = Q[m];
   }
 }
 
 __device__ __forceinline__ StreamConst stream_const(const VelConst<float>& v, bool sy) {
   StreamConst c;
-  c.cp = dup2(sy ? v.cy : 0.0f);
-  c.cm = dup2(sy ? 0.0f : -v.cy);
-  c.b0 = dup2(sy ? v.qy0 : -v.qy0);
-  c.b1 = sy ? v.qy1 : -v.qy1;
+  c.cy = dup2(sy ? v.cy : -v.cy);
+  c.b0 = dup2(v.by0);
+  c.b1 = v.by1;
   return c;
 }
 
@@ -476,7 +477,7 @@ struct Stager {
   Split<ST> split;   // of the segment
   int mixed = 0;     // the lanes' copies may still be in the slots
   int xa = 0, xb = 0;  // without tensor maps: the lane's two lattice columns
-  const int q;
+  const int q;       // quadrants 0 and 1 (s_y > 0) stage one row behind the others
   ST* const base;    // the warp's slots
   const unsigned base_u, full;  // their address and their mbarriers'
 
@@ -487,7 +488,7 @@ struct Stager {
   }
   __device__ __forceinline__ void open() {
     left = feed.next(seg) ? seg.batches() : 0;
-    r0 = seg.ys - RPI;
+    r0 = seg.ys - RPI - (q < 2);
     x0 = seg.strip * TW - XOFF - L::SOFF;
     split = split_of<ST, VEC>(x0, feed.args(seg).Lx);
     if (!VEC && left > 0) {
@@ -572,7 +573,7 @@ __device__ __forceinline__ void advect_role(Feed feed, const StreamSmem<ST>& S, 
     const Split<ST> split = split_of<ST, VEC>(seg.strip * TW - XOFF - L::SOFF, P.Lx);
     const ST* const src0 = stager.base + split.at(h, L::SOFF + col);
     const int pitch = split.pitch(L::SOFF + col);
-    int n = seg.ys - RPI;  // first staged row of the half batch
+    int n = seg.ys - RPI - sy;  // first staged row of the half batch
 #pragma unroll 1
     for (int it = seg.batches(); it > 0; --it, ++g) {
       // the ring rows this batch writes were last read by the collision of g - 2
@@ -610,7 +611,7 @@ __device__ __forceinline__ void advect_role(Feed feed, const StreamSmem<ST>& S, 
         if (edge) {  // ... also after the advection
 #pragma unroll 1
           for (int r = 0; r < SR; ++r) {
-            const int a = n - 2 + r;
+            const int a = n - 2 + sy + r;
             if (a >= 0 && a < Ly) continue;
             float* d = dst + r * (16 * REG);
             const float ga = a < 0 ? va.gbot : va.gtop, gb = a < 0 ? vb.gbot : vb.gtop;
@@ -693,19 +694,12 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
           if ((in0 && !(rho.x > 0.0f && rho.x < 1e30f)) ||
               (in1 && !(rho.y > 0.0f && rho.y < 1e30f)))
             atomicOr(P.err, 1u);
-          float2 s1 = dup2(P.one_m_omega), rw = rho, cr = dup2(0.0f);
-          if (P.reservoir) {
-            // outside R_BC the node is rescaled to rho_ext, s = rho_ext / rho
-            const float dx = (float)x4 - P.cxc, dy = (float)c - P.cyc;
-            const auto rescale = [&](float& a, float& b, float& e, float i) {
-              const float s = P.rho_ext * i;
-              a *= s;
-              b *= s;  // (not rho_ext: s must scale mass and momentum alike)
-              e = P.rho_ref * (s - 1.0f) * (REGU ? 1.0f : P.irho_ext);
-            };
-            if (dx * dx + dy * dy > P.rbc2) rescale(s1.x, rw.x, cr.x, ir.x);
-            if ((dx + 1.0f) * (dx + 1.0f) + dy * dy > P.rbc2) rescale(s1.y, rw.y, cr.y, ir.y);
-          }
+          // outside R_BC the density reservoir rescales the node to rho_ext, s = rho_ext / rho
+          const float dx0 = (float)x4 - P.cxc, dx1 = (float)(x4 + 1) - P.cxc, dy = (float)c - P.cyc;
+          float2 s = dup2(1.0f);
+          if (P.reservoir && dx0 * dx0 + dy * dy > P.rbc2) s.x = P.rho_ext * ir.x;
+          if (P.reservoir && dx1 * dx1 + dy * dy > P.rbc2) s.y = P.rho_ext * ir.y;
+          const float2 rw = mul2(s, rho);  // the density after the step
           const float* fsrc = S.fs + frow * (16 * REG) + cc;
           auto load = [&](int k) { return *reinterpret_cast<const float2*>(fsrc + k * REG); };
           // plane k of the pair: one widening multiply-add per store
@@ -715,21 +709,27 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
             return reinterpret_cast<ST*>(
                 dst0 + (unsigned long long)(unsigned)P.plane * (unsigned)(k * sizeof(ST)));
           };
-          if constexpr (VEC) {  // Lx is even: a pair is inside or outside
-            pair_collide<Pair32, REGU>(
-                P, C, load,
-                [&](int k, float2 o) {
-                  if (in0) store_pair(at(k), o);
-                },
-                drho, rho, ir, u, v, gx, gy, s1, rw, cr);
+          const auto put = [&](int k, float2 o) {
+            if constexpr (VEC) {  // Lx is even: a pair is inside or outside
+              if (in0) store_pair(at(k), o);
+            } else {
+              if (in0) at(k)[0] = to_store<ST, float>(o.x);
+              if (in1) at(k)[1] = to_store<ST, float>(o.y);
+            }
+          };
+          if constexpr (REGU) {
+            pair_collide<Pair32, REGU>(P, C, load, put, drho, rho, ir, u, v, gx, gy,
+                                       mul2(dup2(P.one_m_omega), s), rw,
+                                       mul2(dup2(P.rho_ref), sub2(s, dup2(1.0f))));
+          } else if (P.reservoir) {
+            // the stored deviation becomes s f + w_k rho_ref (s - 1)
+            const float2 s_1 = sub2(s, dup2(1.0f));
+            group_collide(P, C, load, [&](int k, float2 o) {
+              const int grp = k >> 2, cl = grp == 0 ? 0 : (grp == 3 ? 2 : 1);
+              put(k, fma2(s, o, mul2(dup2(P.w[cl] * P.rho_ref), s_1)));
+            }, drho, rho, ir, u, v, gx, gy);
           } else {
-            pair_collide<Pair32, REGU>(
-                P, C, load,
-                [&](int k, float2 o) {
-                  if (in0) at(k)[0] = to_store<ST, float>(o.x);
-                  if (in1) at(k)[1] = to_store<ST, float>(o.y);
-                },
-                drho, rho, ir, u, v, gx, gy, s1, rw, cr);
+            group_collide(P, C, load, put, drho, rho, ir, u, v, gx, gy);
           }
           if (DIAG) post = make_float2(in0 ? rw.x : -1.0f, in1 ? rw.y : -1.0f);
         }
