@@ -60,6 +60,9 @@ struct StreamRegs {
   static_assert(ADVECT + COLLIDE == 2 * LAUNCH, "");
 };
 constexpr unsigned WAIT_NS = 1000000000u;
+// Fused diagnostics: nodes whose mass a lane adds up in FP32 before the sum goes to FP64
+// (the rounding of a sum grows with its terms).
+constexpr int DIAG_RUN = 64;
 
 template <typename ST>
 struct StreamLayout {
@@ -769,6 +772,11 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
             }
           }
         }
+      }
+      if (DIAG && nseg >= DIAG_RUN - 1) {
+        dmass += (double)dseg + (double)P.rho_ref * (double)nseg;
+        dseg = 0.0f;
+        nseg = 0;
       }
       role_arrive(BAR_FREE + (g & 1));
       ring = ring >= SFR - RPI ? ring - (SFR - RPI) : ring + RPI;
