@@ -287,14 +287,14 @@ int lbm_batch_get_info(lbm_batch* b, lbm_batch_info* out);
 
 /* Launch geometry of the handle's fused step kernel (no counterpart in the
  * paper: for tuning, benchmarking and tests).
- *   grid          CTAs of the persistent launch (SMs x resident CTAs at most; a
- *                 launch that would leave SMs idle has its items handed out in
- *                 parts of 8 or 4 rows)
- *                 (FP64: of the advection kernel, as the next two)
+ *   grid          CTAs of the persistent launch (SMs x resident CTAs at most;
+ *                 FP64: of the advection kernel, as the next two)
  *   threads       threads per CTA
  *   smem_bytes    dynamic shared memory per CTA
  *   strips        strips of 56 output columns across x
- *   row_block     rows per work item (work items = strips x row blocks)
+ *   row_block     rows per row block (work items = strips x row blocks, until
+ *                 lbm_set_launch or lbm_tune chooses a geometry divided into
+ *                 parts of 8 or 4 rows where whole blocks would leave SMs idle)
  *   tensor_copies 1 when f^n rows are staged with tensor (TMA) copies, 0 when
  *                 they are loaded value by value (Lx not a multiple of 4, or of
  *                 8 for FP16 storage, or Lx < 72)
@@ -315,7 +315,7 @@ int lbm_get_kernel_info(const lbm_handle* h, lbm_kernel_info* out);
 int lbm_tune(lbm_handle* h, int32_t steps_per_trial, lbm_kernel_info* out);
 
 /* Set the launch geometry explicitly (e.g. one that lbm_tune chose earlier for
- * the same lattice size): row blocks of row_block rows, at most ctas_per_sm
+ * the same lattice size): row blocks of row_block rows (never divided), at most ctas_per_sm
  * resident CTAs per SM (0: as many as the kernel's resources allow on this
  * device).  Results do not depend on it.  No counterpart in the paper.
  * Returns LBM_ERR_INVALID_ARG for a null handle, row_block < 1 or

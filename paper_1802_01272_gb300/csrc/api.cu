@@ -34,6 +34,7 @@ struct lbm_handle {
   int grid = 0;
   int nstrip = 0;
   int row_block = 256;
+  bool parts = true;  // row blocks may be handed out in parts (see apply_geometry)
   bool vec = false;
   size_t smem = 0;
   double xi[16][2], w[16];
@@ -389,14 +390,16 @@ int grid_for(const lbm_handle* h, long long rb, int nsm, int ctas) {
   return (int)(want < gmax ? want : gmax);
 }
 
-// Row blocks of rb rows on at most ctas CTAs per SM.
-void apply_geometry(lbm_handle* h, int rb, int nsm, int ctas) {
+// Row blocks of rb rows on at most ctas CTAs per SM; parts: blocks may be divided (a
+// geometry chosen here, not one that was asked for).
+void apply_geometry(lbm_handle* h, int rb, int nsm, int ctas, bool parts) {
   h->row_block = rb;
   h->a64.sub = pick_sub_f64(h->p.Ly, h->nstrip, rb, nsm);
   h->grid = grid_for(h, rb, nsm, ctas);
   h->a32.row_block = h->a64.row_block = rb;
   h->a32.items = h->a64.items = (long long)((h->p.Ly + rb - 1) / rb) * h->nstrip;
-  if (h->elem == 8) return;
+  h->parts = parts;
+  if (h->elem == 8 || !parts) return;
   // A launch that leaves SMs without a CTA is bound by one item's latency: its blocks
   // are handed out in parts of 8 or 4 rows while there is an SM for each (128 x 8:
   // 7.3 us per step in one part of 8 rows per strip, 6.0 in two of 4).
@@ -514,7 +517,7 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
     fill_step_args<double>(h, h->a64);
   else
     fill_step_args<float>(h, h->a32);
-  apply_geometry(h, h->row_block, nsm, occ);
+  apply_geometry(h, h->row_block, nsm, occ, true);
   h->a32.tma_in = h->a64.tma_in = tin;
   AuxArgs& x = h->aux;
   x.Lx = p->Lx;
@@ -750,7 +753,7 @@ int lbm_set_launch(lbm_handle* h, int32_t row_block, int32_t ctas_per_sm) {
   if (nsm < 1 || occ < 1) return set_err(h, LBM_ERR_CUDA);
   if (ctas_per_sm > occ) return LBM_ERR_INVALID_ARG;
   if (ctas_per_sm == 0) ctas_per_sm = occ;
-  apply_geometry(h, row_block, nsm, ctas_per_sm);
+  apply_geometry(h, row_block, nsm, ctas_per_sm, false);
   drop_graphs(h);  // built for the old geometry
   return LBM_OK;
 }
@@ -767,11 +770,10 @@ int lbm_tune(lbm_handle* h, int32_t steps_per_trial, lbm_kernel_info* out) {
     if (e0) cudaEventDestroy(e0);
     return set_err(h, LBM_ERR_CUDA);
   }
-  auto apply = [&](int rb, int ctas) { apply_geometry(h, rb, nsm, ctas); };
-  // one trial: n real steps with geometry (rb, ctas), GPU time in ms
+  // one trial: n real steps with geometry (rb, ctas, parts), GPU time in ms
   int r = LBM_OK;
-  auto trial = [&](int rb, int ctas, int n, float* ms) -> bool {
-    apply(rb, ctas);
+  auto trial = [&](int rb, int ctas, bool parts, int n, float* ms) -> bool {
+    apply_geometry(h, rb, nsm, ctas, parts);
     cudaEventRecord(e0, h->stream);
     for (int s = 0; s < n; ++s) {
       const cudaError_t e = launch_one(h, h->cur, lim);
@@ -789,35 +791,39 @@ int lbm_tune(lbm_handle* h, int32_t steps_per_trial, lbm_kernel_info* out) {
     return true;
   };
   const int cur_rb = h->row_block;
+  const bool cur_parts = h->parts;
   int cur_c = (int)((h->grid + nsm - 1) / nsm);
   cur_c = cur_c < 1 ? 1 : (cur_c > occ ? occ : cur_c);
   // the current geometry sets the trial length: at least ~1 ms of GPU time
   float ms = 0.0f;
   int steps = steps_per_trial;
-  if (trial(cur_rb, cur_c, steps_per_trial, &ms) && ms > 0.0f && ms < 1.0f) {
+  if (trial(cur_rb, cur_c, cur_parts, steps_per_trial, &ms) && ms > 0.0f && ms < 1.0f) {
     const float want = steps_per_trial / ms;
     steps = want > 1000.0f ? 1000 : (int)want + 1;
   }
   float best = 0.0f;
   int best_rb = cur_rb, best_c = cur_c;
-  if (r == LBM_OK && trial(cur_rb, cur_c, steps, &best)) {
+  bool best_parts = cur_parts;
+  if (r == LBM_OK && trial(cur_rb, cur_c, cur_parts, steps, &best)) {
+    const bool divided = h->elem != 8 && h->a32.row_block != cur_rb;
     const int rbs[] = {16, 32, 64, 96, 128, 192, 256, 384, 512, 1024};
     for (int ctas = 1; ctas <= occ && r == LBM_OK; ++ctas) {
       for (int rb : rbs) {
         if (rb > 16 && rb >= 2 * h->p.Ly) break;  // one block covers the lattice already
-        if (rb == cur_rb && ctas == cur_c) continue;
-        if (!trial(rb, ctas, steps, &ms)) break;
+        if (rb == cur_rb && ctas == cur_c && !divided) continue;
+        if (!trial(rb, ctas, false, steps, &ms)) break;
         if (ms < best) {
           best = ms;
           best_rb = rb;
           best_c = ctas;
+          best_parts = false;
         }
       }
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  apply(best_rb, best_c);
+  apply_geometry(h, best_rb, nsm, best_c, best_parts);
   drop_graphs(h);  // built for the old geometry
   if (out) lbm_get_kernel_info(h, out);
   return r;

@@ -37,3 +37,41 @@ def test_fused_mass_is_as_exact_for_any_row_block(P, precision, Lx, Ly, row_bloc
                 exact = M.step_diag(1, 0.5)["mass"] * Ly / 4
     excess = exact - Lx * Ly
     assert abs(fused["mass"] - exact) <= 64 * 2.0 ** -24 * excess
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+def test_set_launch_is_what_runs_on_a_small_lattice(P, precision):
+    """A geometry that was asked for is launched and reported: one CTA per strip and row block
+    (three strips of 56 columns here, fewer items than SMs).  The state does not depend on it."""
+    prec = {"fp32": P.LBM_FP32_SHIFTED, "fp16": P.LBM_FP16_SHIFTED}[precision]
+    p = P.Params(Lx=128, Ly=64, rho_ref=1.0, precision=prec)
+    y, x = np.mgrid[0:64, 0:128]
+    rho = 1.0 + 0.01 * (((x * 31 + y * 17) % 29) / 29.0)
+    want = None
+    for row_block, ctas in ((0, 0), (16, 1), (24, 0), (32, 1), (64, 2), (8, 1), (4, 1)):
+        with P.Lattice(p) as L:
+            if row_block:
+                k = L.set_launch(row_block, ctas)
+                assert k["row_block"] == row_block and k["grid"] == 3 * -(-64 // row_block), k
+            L.init_rho_u(rho, 0.02 * rho, -0.01 * rho)
+            L.step(35)
+            f = L.get_f()
+            if row_block:
+                assert L.kernel_info() == k
+        want = f if want is None else want
+        assert np.array_equal(f, want)
+
+
+def test_tune_keeps_a_geometry_it_timed(P):
+    """lbm_tune on a small lattice: either the geometry it began with or one of its candidates,
+    which are launched undivided; set_launch with the reported row blocks then runs the same."""
+    p = P.Params(Lx=128, Ly=64, rho_ref=1.0)
+    with P.Lattice(p) as L:
+        L.init_rho_u(np.ones((64, 128)), np.zeros((64, 128)), np.zeros((64, 128)))
+        begun = L.kernel_info()
+        k = L.tune(2)
+        assert k == begun or k["grid"] == 3 * -(-64 // k["row_block"]), (begun, k)
+        k = L.set_launch(16, 1)
+        assert k["grid"] == 12
+        t = L.tune(2)
+        assert t["grid"] == 3 * -(-64 // t["row_block"]), t
