@@ -319,8 +319,9 @@ int lbm_tune(lbm_handle* h, int32_t steps_per_trial, lbm_kernel_info* out);
  * resident CTAs per SM (0: as many as the kernel's resources allow on this
  * device).  Results do not depend on it.  No counterpart in the paper.
  * Returns LBM_ERR_INVALID_ARG for a null handle, row_block < 1 or
- * ctas_per_sm < 0 or above what the kernel's resources allow; LBM_ERR_CUDA if
- * the device cannot be queried. */
+ * ctas_per_sm < 0 or above what the kernel's resources allow (FP32 and FP16:
+ * above 3; the regularised kernel then runs with as many as fit); LBM_ERR_CUDA
+ * if the device cannot be queried. */
 int lbm_set_launch(lbm_handle* h, int32_t row_block, int32_t ctas_per_sm);
 
 /* Measured compute peaks of the current device (no counterpart in the paper:

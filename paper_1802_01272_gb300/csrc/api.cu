@@ -751,8 +751,11 @@ int lbm_set_launch(lbm_handle* h, int32_t row_block, int32_t ctas_per_sm) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
   const int occ = occupancy(h);
   if (nsm < 1 || occ < 1) return set_err(h, LBM_ERR_CUDA);
-  if (ctas_per_sm > occ) return LBM_ERR_INVALID_ARG;
-  if (ctas_per_sm == 0) ctas_per_sm = occ;
+  // Three in FP32 and FP16 whatever the collision: the regularised kernel, which has two
+  // resident, takes a geometry of the plain one.
+  const int most = h->elem == 8 || occ > StreamRegs<false>::CTAS ? occ : StreamRegs<false>::CTAS;
+  if (ctas_per_sm > most) return LBM_ERR_INVALID_ARG;
+  if (ctas_per_sm == 0 || ctas_per_sm > occ) ctas_per_sm = occ;
   apply_geometry(h, row_block, nsm, ctas_per_sm, false);
   drop_graphs(h);  // built for the old geometry
   return LBM_OK;

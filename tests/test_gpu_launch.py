@@ -75,3 +75,19 @@ def test_tune_keeps_a_geometry_it_timed(P):
         assert k["grid"] == 12
         t = L.tune(2)
         assert t["grid"] == 3 * -(-64 // t["row_block"]), t
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+@pytest.mark.parametrize("regularize", [0, 1])
+@pytest.mark.parametrize("Lx", [128, 113])
+def test_set_launch_takes_three_ctas_per_sm(P, precision, regularize, Lx):
+    """One, two or three CTAs per SM are accepted for every FP32 and FP16 kernel, four are not."""
+    prec = {"fp32": P.LBM_FP32_SHIFTED, "fp16": P.LBM_FP16_SHIFTED}[precision]
+    with P.Lattice(P.Params(Lx=Lx, Ly=4096, precision=prec, regularize=regularize)) as L:
+        for ctas in (1, 2, 3):
+            assert L.set_launch(4, ctas)["row_block"] == 4
+        with pytest.raises(Exception):
+            L.set_launch(4, 4)
+        L.init_rho_u(np.ones((4096, Lx)), np.zeros((4096, Lx)), np.zeros((4096, Lx)))
+        L.step(2)
+        L.sync()
