@@ -91,3 +91,23 @@ def test_set_launch_takes_three_ctas_per_sm(P, precision, regularize, Lx):
         L.init_rho_u(np.ones((4096, Lx)), np.zeros((4096, Lx)), np.zeros((4096, Lx)))
         L.step(2)
         L.sync()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("row_block", [41, 1025, 2 ** 31 - 1])
+def test_row_blocks_higher_than_the_lattice(P, precision, row_block):
+    """Any row block from the lattice's height on is one block: the state is the default's."""
+    prec = {"fp64": P.LBM_FP64, "fp32": P.LBM_FP32_SHIFTED, "fp16": P.LBM_FP16_SHIFTED}[precision]
+    p = P.Params(Lx=130, Ly=41, rho_ref=1.0, precision=prec)
+    y, x = np.mgrid[0:41, 0:130]
+    rho = 1.0 + 0.01 * (((x * 31 + y * 17) % 29) / 29.0)
+    out = []
+    for rb in (0, row_block):
+        with P.Lattice(p) as L:
+            if rb:
+                assert L.set_launch(rb, 1)["row_block"] == rb
+            L.init_rho_u(rho, 0.02 * rho, -0.01 * rho)
+            L.step(5)
+            L.sync()
+            out.append(L.get_f())
+    assert np.array_equal(*out)
