@@ -225,7 +225,6 @@ void fill_step_args(lbm_handle* h, StepArgs<T>& a) {
     VelConst<T>& v = a.v[k];
     v.xi_x = (T)x;
     v.xi_y = (T)y;
-    v.w = (T)h->w[k];
     // CTU2 per node (Sec. II C 2 collected): with Z(j) = f - c_x (f - f(i - s_x))
     // - 2 lam hx dS^x(j), the update is Z(j) + c_y (Z(j - s_y) - Z(j))
     // - 2 lam hy [(1 - c_x) dS^y(i) + c_x dS^y(i - s_x)] on the kernels'

@@ -277,8 +277,6 @@ __global__ void hist_kernel(const AuxArgs a, const S* f, int nbins, double lo, d
 
 unsigned grid_for(long long n) { return (unsigned)((n + BS - 1) / BS); }
 
-}  // namespace
-
 // Whether nodes can be taken two at a time: an even number of them, and the caller's
 // fields (whose alignment is only that of a double) on 16-byte boundaries.
 bool two_nodes(const AuxArgs& a, const void* x, const void* y, const void* z) {
@@ -296,6 +294,8 @@ cudaError_t by_storage(const AuxArgs& a, const void* f, F fn) {
   }
   return cudaGetLastError();
 }
+
+}  // namespace
 
 cudaError_t launch_init_feq(const AuxArgs& a, void* f, const double* rho, const double* ux,
                             const double* uy, cudaStream_t s) {

@@ -32,7 +32,7 @@ constexpr int WARM = 2;         // batches of a segment before its first output 
 // Per-velocity constants, computed on the host in FP64 and rounded to T.
 template <typename T>
 struct VelConst {
-  T xi_x, xi_y, w;
+  T xi_x, xi_y;
   T cx, cy;                 // Courant numbers |xi_x| dt/ds, |xi_y| dt/ds
   T ax;                     // lam |xi_x| (1 - cx): weight of the x-difference of half-limited S^x
   T qy0, qy1;               // FP64: (1 - cy) (1 - cx), (1 - cy) cx: weights of the S^y terms per unit of cy
