@@ -60,9 +60,6 @@ struct StreamRegs {
   static_assert(ADVECT + COLLIDE == 2 * LAUNCH, "");
 };
 constexpr unsigned WAIT_NS = 1000000000u;
-// Fused diagnostics: nodes whose mass a lane adds up in FP32 before the sum goes to FP64
-// (the rounding of a sum grows with its terms).
-constexpr int DIAG_RUN = 64;
 
 template <typename ST>
 struct StreamLayout {
@@ -82,11 +79,12 @@ struct StreamSmem {
   float *drho, *phi;        // [SMR][MPP]
   float *ux, *uy;           // [SFR][MPP]
   unsigned long long* dsums;    // [6] fused diagnostics: per-CTA bubble-site sums
+  double* mass;                 // [128] and each collide thread's sum of rho - rho_ref
   unsigned long long *full;     // [4][SNS] a staged batch has landed
   int* abort;                   // [4] a bounded wait of this advect warp timed out
   static constexpr size_t bytes() {
     return 128 + sizeof(ST) * L::STAGE + 4 * (SFR * 16 * REG + 2 * (SMR + SFR) * MPP) +
-           8 * (6 + 4 * SNS) + 16;
+           8 * (6 + 128 + 4 * SNS) + 16;
   }
   __device__ explicit StreamSmem(unsigned char* raw) {
     raw += (128u - (smem_u32(raw) & 127u)) & 127u;  // tensor copies want 128-byte aligned tiles
@@ -97,10 +95,12 @@ struct StreamSmem {
     ux = phi + SMR * MPP;
     uy = ux + SFR * MPP;
     dsums = reinterpret_cast<unsigned long long*>(uy + SFR * MPP);
-    full = dsums + 6;
+    mass = reinterpret_cast<double*>(dsums + 6);
+    full = dsums + 6 + 128;
     abort = reinterpret_cast<int*>(full + 4 * SNS);
   }
   __device__ void init() const {
+    if (threadIdx.x < 128) mass[threadIdx.x] = 0.0;
     if (threadIdx.x == 0) {
       for (int t = 0; t < 6; ++t) dsums[t] = 0ULL;
       for (int b = 0; b < 4; ++b) abort[b] = 0;
@@ -652,8 +652,6 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
     const StepArgs<float>& P = feed.args(seg);
     const int nit = seg.batches(), x4 = seg.strip * TW + 2 * lane;
     const NodeConst<Pair32> C(P);
-    float dseg = 0.0f;
-    int nseg = 0;
 #pragma unroll 1
     for (int it = 0; it < nit; ++it, ++g) {
       role_wait(BAR_FULL + (g & 1));
@@ -677,7 +675,7 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
       if (it >= WARM) {
         collide_barrier();
         const int c = c0 + w;  // this warp's row
-        float2 post = dup2(-1.0f);
+        int bubble = 0;          // fused diagnostics: which of the two nodes are bubble sites
         if (lane < TW / 2) {
           const float *ph[5], *dq[5];
 #pragma unroll
@@ -706,6 +704,16 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
           if (P.reservoir && dx0 * dx0 + dy * dy > P.rbc2) s.x = P.rho_ext * ir.x;
           if (P.reservoir && dx1 * dx1 + dy * dy > P.rbc2) s.y = P.rho_ext * ir.y;
           const float2 rw = mul2(s, rho);  // the density after the step
+          if (DIAG) {
+            // The mass goes to FP64 row by row, in shared memory: a sum of many rows would
+            // round too much in FP32, and held in registers it costs the loop spills (6144^2
+            // with fused diagnostics 1359 -> 1260 us).  A density that is not one (flagged
+            // above) counts as none.
+            const bool ok0 = in0 && rw.x >= 0.0f, ok1 = in1 && rw.y >= 0.0f;
+            S.mass[threadIdx.x & 127] += (double)((in0 ? (ok0 ? rw.x : 0.0f) - P.rho_ref : 0.0f) +
+                                                  (in1 ? (ok1 ? rw.y : 0.0f) - P.rho_ref : 0.0f));
+            bubble = (ok0 && rw.x < P.diag_thr ? 1 : 0) | (ok1 && rw.y < P.diag_thr ? 2 : 0);
+          }
           const float* fsrc = S.fs + frow * (16 * REG) + cc;
           auto load = [&](int k) { return *reinterpret_cast<const float2*>(fsrc + k * REG); };
           // plane k of the pair: one widening multiply-add per store
@@ -737,53 +745,38 @@ __device__ __forceinline__ void collide_role(Feed feed, const StreamSmem<ST>& S,
           } else {
             group_collide(P, C, load, put, drho, rho, ir, u, v, gx, gy);
           }
-          if (DIAG) post = make_float2(in0 ? rw.x : -1.0f, in1 ? rw.y : -1.0f);
         }
-        if (DIAG) {  // fused diagnostics: mass per thread, bubble sites per warp
+        if (DIAG && __ballot_sync(0xffffffffu, bubble != 0)) {  // bubble sites are rare
           unsigned long long a[6] = {0, 0, 0, 0, 0, 0};
-          bool any = false;
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            const float p = e ? post.y : post.x;
-            if (p >= 0.0f) {
-              dseg += p - P.rho_ref;
-              ++nseg;
-              if (p < P.diag_thr) {
-                const unsigned long long i = (unsigned long long)(x4 + e), j = (unsigned long long)c;
-                any = true;
-                a[0] += 1;
-                a[1] += i;
-                a[2] += j;
-                a[3] += i * i;
-                a[4] += i * j;
-                a[5] += j * j;
-              }
+            if (bubble >> e & 1) {
+              const unsigned long long i = (unsigned long long)(x4 + e), j = (unsigned long long)c;
+              a[0] += 1;
+              a[1] += i;
+              a[2] += j;
+              a[3] += i * i;
+              a[4] += i * j;
+              a[5] += j * j;
             }
           }
-          if (__ballot_sync(0xffffffffu, any)) {  // bubble sites are rare: sum them only here
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
+          for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-              for (int t = 0; t < 6; ++t) a[t] += __shfl_down_sync(0xffffffffu, a[t], o);
-            }
-            if (lane == 0) {
+            for (int t = 0; t < 6; ++t) a[t] += __shfl_down_sync(0xffffffffu, a[t], o);
+          }
+          if (lane == 0) {
 #pragma unroll
-              for (int t = 0; t < 6; ++t) atomicAdd(&S.dsums[t], a[t]);
-            }
+            for (int t = 0; t < 6; ++t) atomicAdd(&S.dsums[t], a[t]);
           }
         }
-      }
-      if (DIAG && nseg >= DIAG_RUN - 1) {
-        dmass += (double)dseg + (double)P.rho_ref * (double)nseg;
-        dseg = 0.0f;
-        nseg = 0;
       }
       role_arrive(BAR_FREE + (g & 1));
       ring = ring >= SFR - RPI ? ring - (SFR - RPI) : ring + RPI;
       mring = mring == SMR - RPI ? 0 : mring + RPI;
     }
-    if (DIAG) dmass += (double)dseg + (double)P.rho_ref * (double)nseg;
   }
+  if (DIAG) dmass = S.mass[threadIdx.x & 127];
 }
 
 template <int FROM, int TO>
@@ -825,10 +818,12 @@ __global__ void __launch_bounds__(NT, StreamRegs<REGU>::CTAS)
   if (VEC && threadIdx.x == 0) prefetch_map(maps.m);
   S.init();
   previous_step_done();
-  double dmass = 0.0;  // fused diagnostics: this thread's mass over all its segments
+  // fused diagnostics: rho - rho_ref of this thread's nodes, and rho_ref of every node once
+  double dmass = 0.0;
   stream_roles<ORDER, LIM, ST, VEC, DIAG, REGU>(SingleFeed(P, maps), S, dmass);
   if (DIAG) {
     // one warp sum and one global add per warp for the mass
+    if (blockIdx.x == 0 && threadIdx.x == 0) dmass = (double)P.rho_ref * (double)P.plane;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dmass += __shfl_down_sync(0xffffffffu, dmass, o);
     if ((threadIdx.x & 31) == 0 && dmass != 0.0) atomicAdd(P.diag_mass, dmass);
