@@ -290,14 +290,14 @@ int lbm_batch_get_info(lbm_batch* b, lbm_batch_info* out);
  *   grid          CTAs of the persistent launch (SMs x resident CTAs at most;
  *                 FP64: of the advection kernel, as the next two)
  *   threads       threads per CTA
- *   smem_bytes    dynamic shared memory per CTA
+ *   smem_bytes    dynamic shared memory per CTA (FP64: 0, it is static)
  *   strips        strips of 56 output columns across x
  *   row_block     rows per row block (work items = strips x row blocks, until
  *                 lbm_set_launch or lbm_tune chooses a geometry divided into
  *                 parts of 8 or 4 rows where whole blocks would leave SMs idle)
  *   tensor_copies 1 when f^n rows are staged with tensor (TMA) copies, 0 when
  *                 they are loaded value by value (Lx not a multiple of 4, or of
- *                 8 for FP16 storage, or Lx < 72)
+ *                 8 for FP16 storage, or Lx < 68, 72 for FP16 storage)
  * Returns LBM_ERR_INVALID_ARG for a null argument; the handle is not touched. */
 typedef struct lbm_kernel_info {
   int32_t grid, threads, smem_bytes, strips, row_block, tensor_copies;

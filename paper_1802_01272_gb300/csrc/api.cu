@@ -40,8 +40,7 @@ struct lbm_handle {
   double xi[16][2], w[16];
   StepArgs<float> a32;
   StepArgs<double> a64;
-  // tensor maps of the step from f[c] to f[1 - c]: loads of f[c] (RPI-row and
-  // 1-row staging boxes), stores of output tiles into f[1 - c]
+  // tensor maps of f[c], which a step stages its rows by (see RowMaps)
   RowMaps tmap[2];
   // CUDA graphs of GRAPH_STEPS consecutive steps starting from f[0] / f[1]
   // (built on first use, rebuilt when the launch geometry changes)
@@ -502,8 +501,8 @@ int lbm_create(const lbm_params* p, void* cuda_stream, lbm_handle** out) {
   }
   h->vec = tin;  // else every strip is staged value by value
 
-  // launch geometry: strips of TW output columns, rows split evenly over a
-  // persistent grid of (SMs x resident CTAs), at least 48 rows per CTA
+  // launch geometry: strips of TW output columns and blocks of rows on a
+  // persistent grid of at most SMs x resident CTAs (see pick_row_block)
   h->nstrip = (p->Lx + TW - 1) / TW;
   h->smem = h->elem == 8 ? 0 : step_smem_bytes(h->elem);
   const int occ = occupancy(h);

@@ -209,8 +209,8 @@ int lbm_batch_create(size_t max_bytes, int32_t chunk_steps, void* cuda_stream, l
   int nsm = 0;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess)
     return LBM_ERR_CUDA;
-  // the batched kernel's resident CTAs per SM (CTU2 + MC, FP32 storage), two
-  // work items of 96 rows x 56 columns each
+  // nodes that fill the GPU: 2 x 96 x 56 for each resident CTA of the batched kernel
+  // (CTU2 + MC, FP32 storage)
   int occ = ctulbm::step_batch_occupancy_f32(2, 0, false, ctulbm::step_smem_bytes(4));
   if (occ < 1) occ = 2;
   b->fill_nodes = (long long)nsm * occ * 2 * 96 * 56;

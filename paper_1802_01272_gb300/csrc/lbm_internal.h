@@ -40,7 +40,7 @@ inline cudaError_t launch_dependent(const void* fn, unsigned grid, unsigned thre
 }
 
 // One fused step kernel: returns cudaSuccess or the launch error.  `vec`: the
-// lattice has tensor maps (`maps`, for a.fin and a.fout) and stages by them.
+// lattice has tensor maps (`maps`, those of a.fin) and stages by them.
 cudaError_t launch_step_f32(const StepArgs<float>& a, const RowMaps& maps, int order, int lim,
                             bool vec, int grid, size_t smem, cudaStream_t s);
 // The FP64 step: advection from `f` into `work`, collision back into `f`; a.fin

@@ -15,7 +15,8 @@
 //   of the neighbouring group comes from the adjacent lane.  The warp stages its
 //   own four planes, half a batch per slot, by tensor copies that its elected
 //   lane issues as soon as the slot has been read: no other warp touches its
-//   slots, so staging needs no barrier between warps.  A strip at the periodic x
+//   slots, so staging needs no barrier between warps.  The warps with xi_y > 0 stage
+//   one row behind the others (see StreamState).  A strip at the periodic x
 //   seam is staged by two copies, one per side of the seam.  The advected rows
 //   f* go to a ring of ten rows.
 //  warps 4-7 COLLIDE.  Warp 4 + r takes row r of the batch, a lane two
@@ -34,10 +35,11 @@
 // lane hold twice the work (two velocities, two nodes), which halves the loop,
 // barrier and address instructions per node, and replaces three barriers of all
 // warps per batch.  Against one kernel body in which all warps advect, then
-// collide (30 warp instructions per node; now 24): 6144^2 FP32 1.25 -> 1.08
-// ms/step, 2048^2 187 -> 128 us, 1024^2 70 -> 38 us, 1001 x 777 80 -> 35 us, 4096^2
-// FP16 660 -> 504 us.  Measured on the way: two CTAs per SM with 128 registers, as
-// fast at 1024^2 and 7 % slower at 6144^2; the hand-over by polled mbarriers -3 %;
+// collide, with the same operations on every node (30 warp instructions per node;
+// now 25.8): 6144^2 FP32 1.25 -> 1.11 ms/step, 2048^2 187 -> 132 us, 1024^2 70 -> 39
+// us, 1001 x 777 80 -> 38 us, 4096^2 FP16 660 -> 530 us.  Measured on the way, with
+// other sums in the collision (1.08 ms at 6144^2, see group_collide): two CTAs per SM
+// with 128 registers, as fast at 1024^2 and 7 % slower at 6144^2; the hand-over by polled mbarriers -3 %;
 // the row loop unrolled by four instead of two -9 % and one copy of the advection
 // per sign quadrant instead of per sign of xi_x -30 % (instruction fetch); seam
 // strips staged by the lanes' 16-byte copies -17 % at 3584 x 2048 (their CTAs were
