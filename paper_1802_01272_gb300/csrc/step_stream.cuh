@@ -101,8 +101,8 @@ struct StreamSmem {
     full = dsums + 6 + 128;
     abort = reinterpret_cast<int*>(full + 4 * SNS);
   }
-  __device__ void init() const {
-    if (threadIdx.x < 128) mass[threadIdx.x] = 0.0;
+  __device__ __forceinline__ void init(bool diag) const {
+    if (diag && threadIdx.x < 128) mass[threadIdx.x] = 0.0;
     if (threadIdx.x == 0) {
       for (int t = 0; t < 6; ++t) dsums[t] = 0ULL;
       for (int b = 0; b < 4; ++b) abort[b] = 0;
@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(NT, StreamRegs<REGU>::CTAS)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const StreamSmem<ST> S(smem_raw);
   if (VEC && threadIdx.x == 0) prefetch_map(maps.m);
-  S.init();
+  S.init(DIAG);
   previous_step_done();
   // fused diagnostics: rho - rho_ref of this thread's nodes, and rho_ref of every node once
   double dmass = 0.0;
@@ -841,7 +841,7 @@ __global__ void __launch_bounds__(NT, StreamRegs<REGU>::CTAS)
     stream_batch_kernel(const __grid_constant__ BatchArgs<float> B) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const StreamSmem<float> S(smem_raw);
-  S.init();
+  S.init(false);
   previous_step_done();
   double dmass = 0.0;  // unused: batched launches carry no fused diagnostics
   stream_roles<ORDER, LIM, float, true, false, REGU>(BatchFeed(B), S, dmass);
