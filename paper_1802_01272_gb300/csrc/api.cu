@@ -392,13 +392,13 @@ int grid_for(const lbm_handle* h, long long rb, int nsm, int ctas) {
 // geometry chosen here, not one that was asked for).
 void apply_geometry(lbm_handle* h, int rb, int nsm, int ctas, bool parts) {
   h->row_block = rb;
-  // (a block far higher than the lattice is launched as one of the lattice's height: sums
-  // with it stay within an int)
+  // (a block far higher than the lattice is launched as one of the lattice's height: its
+  // sums with a row stay within an int)
   const int most = h->p.Ly > 1024 ? h->p.Ly : 1024, rows = rb < most ? rb : most;
   h->a64.sub = pick_sub_f64(h->p.Ly, h->nstrip, rows, nsm);
   h->grid = grid_for(h, rows, nsm, ctas);
   h->a32.row_block = h->a64.row_block = rows;
-  h->a32.items = h->a64.items = (long long)((h->p.Ly + rows - 1) / rows) * h->nstrip;
+  h->a32.items = h->a64.items = ((long long)h->p.Ly + rows - 1) / rows * h->nstrip;
   h->parts = parts;
   if (h->elem == 8 || !parts) return;
   // A launch that leaves SMs without a CTA is bound by one item's latency: its blocks
